@@ -136,7 +136,7 @@ __device__ __forceinline__ void cinv_23(cg::cluster_group& cluster, cplx<T>* B, 
     for (int i = 0; i < N; ++i) v[i] = cplx<T>{0, 0};
 #pragma unroll
     for (int c2 = 0; c2 < L; ++c2) v[S::box(c2)] = spec(r, c1_0 + r, c2, c3);
-    Codelet<T, N, +1>::run(v);
+    Codelet<T, N, +1>::template run<S::on()>(v);
 #pragma unroll
     for (int i2 = 0; i2 < N; ++i2) B[D::bidx(r, i2, c3)] = v[i2];
   }
@@ -148,7 +148,7 @@ __device__ __forceinline__ void cinv_23(cg::cluster_group& cluster, cplx<T>* B, 
     for (int i = 0; i < N; ++i) v[i] = cplx<T>{0, 0};
 #pragma unroll
     for (int c3 = 0; c3 < L; ++c3) v[S::box(c3)] = B[D::bidx(r, i2, c3)];
-    Codelet<T, N, +1>::run(v);
+    Codelet<T, N, +1>::template run<S::on()>(v);
 #pragma unroll
     for (int i3 = 0; i3 < N; ++i3) B[D::bidx(r, i2, i3)] = v[i3];
   }
@@ -175,7 +175,7 @@ __device__ __forceinline__ void caxis1(cg::cluster_group& cluster, cplx<T>* cons
       for (int i = 0; i < N; ++i) v[i] = cplx<T>{0, 0};
 #pragma unroll
       for (int c1 = 0; c1 < L; ++c1) v[S::box(c1)] = rb[c1 / D::R][D::bidx(c1 % D::R, i2, i3)];
-      Codelet<T, N, +1>::run(v);
+      Codelet<T, N, +1>::template run<S::on()>(v);
     } else {
 #pragma unroll
       for (int i = 0; i < N; ++i) v[i] = load(i, i2, i3);

@@ -84,89 +84,278 @@ template <typename T, int N, int S> __device__ __forceinline__ cplx<T> twiddle(i
 }
 
 // ---------------------------------------------------------------------------
-// Small butterflies (in place, natural order), exponent sign S.
+// Codelets.  Every transform takes the set IN of its nonzero inputs (bit i: input i) at compile
+// time: the pruned passes feed 17 of 24 (or 13 of 16, ...) values, and IEEE arithmetic keeps
+// x + 0, so a zero that the code does not name costs its additions.  Outputs that nobody reads
+// fall to dead-code elimination.
+//
+// What bounds them: in FP64 the FP64 pipe (1.6 operations per clock and SM), in FP32 the issue
+// slots of the kernels around them.  Measured on one GB300 (3x3x3 FP64 apply / 4x4x4 FP32 apply of
+// the silicon-like cell, 24^3): mixed radix 4 x 3 x 2 with twiddles, zeros unnamed, scalar FP32:
+// 607 / 143.9 ms; as below 501 / 128.1 ms; as below with scalar FP32: - / 136 ms.
+using InSet = unsigned long long;
+template <int N> __host__ __device__ constexpr InSet all_in() { return (N >= 64 ? ~0ull : (1ull << N) - 1ull); }
+
+// FP32 sums of complex values as one packed instruction for both halves (add / fma .f32x2): the
+// lanes do no more per clock (127 against 124 additions per clock and SM measured), but half the
+// instructions are issued
+__device__ __forceinline__ cplx<float> operator+(cplx<float> a, cplx<float> b) {
+  const float2 r = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+  return {r.x, r.y};
+}
+__device__ __forceinline__ cplx<float> operator-(cplx<float> a, cplx<float> b) {
+  const float2 r = __ffma2_rn(make_float2(b.x, b.y), make_float2(-1.f, -1.f), make_float2(a.x, a.y));
+  return {r.x, r.y};
+}
+// a + s b, s real
+template <typename T> __device__ __forceinline__ cplx<T> axpy(T s, cplx<T> b, cplx<T> a) {
+  if constexpr (sizeof(T) == 4) {
+    const float2 r = __ffma2_rn(make_float2(b.x, b.y), make_float2(s, s), make_float2(a.x, a.y));
+    return {r.x, r.y};
+  } else {
+    return {fma(s, b.x, a.x), fma(s, b.y, a.y)};
+  }
+}
+// a + s i b, s real
+template <typename T> __device__ __forceinline__ cplx<T> axpy_i(T s, cplx<T> b, cplx<T> a) {
+  return {fma(-s, b.y, a.x), fma(s, b.x, a.y)};
+}
+// sum and difference of values that may be known zeros
+template <bool ZA, bool ZB, typename T> __device__ __forceinline__ cplx<T> addz(cplx<T> a, cplx<T> b) {
+  if constexpr (ZA && ZB) return a + b;
+  else if constexpr (ZA) return a;
+  else if constexpr (ZB) return b;
+  else return cplx<T>{0, 0};
+}
+template <bool ZA, bool ZB, typename T> __device__ __forceinline__ cplx<T> subz(cplx<T> a, cplx<T> b) {
+  if constexpr (ZA && ZB) return a - b;
+  else if constexpr (ZA) return a;
+  else if constexpr (ZB) return cplx<T>{-b.x, -b.y};
+  else return cplx<T>{0, 0};
+}
+
+// Small butterflies (in place, natural order), exponent sign S, nonzero inputs IN.  The rotations
+// by i and by the real factors of the radix-3, -5 and -8 butterflies are folded into the closing
+// additions as fused multiply-adds: 12, 32 and 52 operations for 3, 5 and 8 points.
 template <typename T, int R, int S> struct Small;
 
 template <typename T, int S> struct Small<T, 2, S> {
-  static __device__ __forceinline__ void run(cplx<T>* z) {
-    cplx<T> a = z[0], b = z[1];
-    z[0] = a + b;
-    z[1] = a - b;
+  template <InSet IN> static __device__ __forceinline__ void run(cplx<T>* z) {
+    constexpr bool A = IN & 1, B = IN & 2;
+    const cplx<T> a = z[0], b = z[1];
+    z[0] = addz<A, B>(a, b);
+    z[1] = subz<A, B>(a, b);
   }
 };
 
 template <typename T, int S> struct Small<T, 3, S> {
-  static __device__ __forceinline__ void run(cplx<T>* z) {
-    const T h = T(0.5), s3 = T(0.86602540378443864676372317075294);   // sqrt(3)/2
-    cplx<T> t1 = z[1] + z[2], t2 = z[1] - z[2];
-    cplx<T> a = z[0];
-    cplx<T> m = a - h * t1;
-    cplx<T> r = mul_si<T, S>(s3 * t2);
-    z[0] = a + t1;
-    z[1] = m + r;
-    z[2] = m - r;
+  template <InSet IN> static __device__ __forceinline__ void run(cplx<T>* z) {
+    constexpr bool A = IN & 1, B = IN & 2, C = IN & 4;
+    const T h = T(0.5), s3 = T(S * 0.86602540378443864676372317075294);   // sqrt(3)/2
+    const cplx<T> a = z[0];
+    if constexpr (!B && !C) {
+      z[1] = a;
+      z[2] = a;
+    } else {
+      const cplx<T> t1 = addz<B, C>(z[1], z[2]), t2 = subz<B, C>(z[1], z[2]);
+      const cplx<T> m = A ? axpy<T>(-h, t1, a) : cplx<T>{-h * t1.x, -h * t1.y};
+      z[0] = addz<A, true>(a, t1);
+      z[1] = axpy_i<T>(s3, t2, m);
+      z[2] = axpy_i<T>(-s3, t2, m);
+    }
   }
 };
 
 template <typename T, int S> struct Small<T, 4, S> {
-  static __device__ __forceinline__ void run(cplx<T>* z) {
-    cplx<T> a = z[0] + z[2], b = z[0] - z[2], c = z[1] + z[3], d = mul_si<T, S>(z[1] - z[3]);
-    z[0] = a + c;
-    z[2] = a - c;
-    z[1] = b + d;
-    z[3] = b - d;
+  template <InSet IN> static __device__ __forceinline__ void run(cplx<T>* z) {
+    constexpr bool A = IN & 1, B = IN & 2, C = IN & 4, D = IN & 8, E = A || C, O = B || D;
+    const cplx<T> a = addz<A, C>(z[0], z[2]), b = subz<A, C>(z[0], z[2]), c = addz<B, D>(z[1], z[3]),
+                  d = mul_si<T, S>(subz<B, D>(z[1], z[3]));
+    z[0] = addz<E, O>(a, c);
+    z[2] = subz<E, O>(a, c);
+    if constexpr (E && O) {   // the rotated difference by halves: no pair to pack
+      z[1] = cplx<T>{b.x + d.x, b.y + d.y};
+      z[3] = cplx<T>{b.x - d.x, b.y - d.y};
+    } else {
+      z[1] = addz<E, O>(b, d);
+      z[3] = subz<E, O>(b, d);
+    }
   }
 };
 
 template <typename T, int S> struct Small<T, 5, S> {
-  static __device__ __forceinline__ void run(cplx<T>* z) {
-    // cos(2 pi/5), cos(4 pi/5), sin(2 pi/5), sin(4 pi/5)
+  template <InSet IN> static __device__ __forceinline__ void run(cplx<T>* z) {
+    constexpr bool A = IN & 1, B1 = IN & 2, B2 = IN & 4, B3 = IN & 8, B4 = IN & 16, P = B1 || B4, Q = B2 || B3;
+    // cos(2 pi/5), cos(4 pi/5), sin(2 pi/5), sin(4 pi/5)/sin(2 pi/5)
     const T c1 = T(0.30901699437494742410229341718282), c2 = T(-0.80901699437494742410229341718282);
-    const T s1 = T(0.95105651629515357211643933337938), s2 = T(0.58778525229247312916870595463907);
-    cplx<T> x0 = z[0];
-    cplx<T> t1 = z[1] + z[4], t2 = z[2] + z[3], t3 = z[1] - z[4], t4 = z[2] - z[3];
-    cplx<T> a1 = x0 + c1 * t1 + c2 * t2, a2 = x0 + c2 * t1 + c1 * t2;
-    cplx<T> b1 = mul_si<T, S>(s1 * t3 + s2 * t4), b2 = mul_si<T, S>(s2 * t3 - s1 * t4);
-    z[0] = x0 + t1 + t2;
-    z[1] = a1 + b1;
-    z[4] = a1 - b1;
-    z[2] = a2 + b2;
-    z[3] = a2 - b2;
+    const T s1 = T(S * 0.95105651629515357211643933337938), r = T(0.61803398874989484820458683436564);
+    const cplx<T> x0 = A ? z[0] : cplx<T>{0, 0};
+    if constexpr (!P && !Q) {
+      z[1] = z[2] = z[3] = z[4] = x0;
+    } else {
+      const cplx<T> t1 = addz<B1, B4>(z[1], z[4]), t2 = addz<B2, B3>(z[2], z[3]), t3 = subz<B1, B4>(z[1], z[4]),
+                    t4 = subz<B2, B3>(z[2], z[3]);
+      cplx<T> a1 = x0, a2 = x0, b1, b2;
+      if constexpr (P) {
+        a1 = axpy<T>(c1, t1, a1);
+        a2 = axpy<T>(c2, t1, a2);
+      }
+      if constexpr (Q) {
+        a1 = axpy<T>(c2, t2, a1);
+        a2 = axpy<T>(c1, t2, a2);
+      }
+      // sin parts over sin(2 pi/5): t3 + r t4 and r t3 - t4
+      if constexpr (P && Q) {
+        b1 = axpy<T>(r, t4, t3);
+        b2 = axpy<T>(r, t3, cplx<T>{-t4.x, -t4.y});
+      } else if constexpr (P) {
+        b1 = t3;
+        b2 = cplx<T>{r * t3.x, r * t3.y};
+      } else {
+        b1 = cplx<T>{r * t4.x, r * t4.y};
+        b2 = cplx<T>{-t4.x, -t4.y};
+      }
+      z[0] = addz<A, true>(x0, addz<P, Q>(t1, t2));
+      z[1] = axpy_i<T>(s1, b1, a1);
+      z[4] = axpy_i<T>(-s1, b1, a1);
+      z[2] = axpy_i<T>(s1, b2, a2);
+      z[3] = axpy_i<T>(-s1, b2, a2);
+    }
   }
 };
 
-__host__ __device__ constexpr int pick_radix(int n) {
-  return (n % 4 == 0) ? 4 : (n % 3 == 0 ? 3 : (n % 2 == 0 ? 2 : (n % 5 == 0 ? 5 : n)));
+template <typename T, int S> struct Small<T, 8, S> {
+  template <InSet IN> static __device__ __forceinline__ void run(cplx<T>* z) {
+    constexpr InSet EV = (IN & 1) | ((IN >> 1) & 2) | ((IN >> 2) & 4) | ((IN >> 3) & 8);
+    constexpr InSet OD = ((IN >> 1) & 1) | ((IN >> 2) & 2) | ((IN >> 3) & 4) | ((IN >> 4) & 8);
+    const T r = T(0.70710678118654752440084436210485);
+    cplx<T> e[4] = {z[0], z[2], z[4], z[6]}, o[4] = {z[1], z[3], z[5], z[7]};
+    if constexpr (EV != 0) Small<T, 4, S>::template run<EV>(e);
+    else e[0] = e[1] = e[2] = e[3] = cplx<T>{0, 0};
+    if constexpr (OD == 0) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) z[k] = z[k + 4] = e[k];
+    } else {
+      Small<T, 4, S>::template run<OD>(o);
+      constexpr bool E = EV != 0;
+      z[0] = addz<E, true>(e[0], o[0]);
+      z[4] = subz<E, true>(e[0], o[0]);
+      const cplx<T> q = mul_si<T, S>(o[2]);
+      z[2] = cplx<T>{e[2].x + q.x, e[2].y + q.y};
+      z[6] = cplx<T>{e[2].x - q.x, e[2].y - q.y};
+      // exp(S i pi/4) o = r u1 and exp(S 3 i pi/4) o = -r u3
+      const cplx<T> u1 = S > 0 ? cplx<T>{o[1].x - o[1].y, o[1].y + o[1].x} : cplx<T>{o[1].x + o[1].y, o[1].y - o[1].x};
+      const cplx<T> u3 = S > 0 ? cplx<T>{o[3].x + o[3].y, o[3].y - o[3].x} : cplx<T>{o[3].x - o[3].y, o[3].y + o[3].x};
+      z[1] = axpy<T>(r, u1, e[1]);
+      z[5] = axpy<T>(-r, u1, e[1]);
+      z[3] = axpy<T>(-r, u3, e[3]);
+      z[7] = axpy<T>(r, u3, e[3]);
+    }
+  }
+};
+
+// Split N = P Q of the codelet for N points.  Coprime factors (the power of 2, of 3 or of 5 taken
+// out first) need no twiddles (Good-Thomas); prime powers beyond the butterflies split by radix 4,
+// 3 or 5 with twiddles.  24 points cost 252 operations this way (3 x 52 + 8 x 12) against 332 for
+// the mixed-radix decimation 4 x 3 x 2 with twiddles.
+__host__ __device__ constexpr bool small_radix(int n) { return n == 2 || n == 3 || n == 4 || n == 5 || n == 8; }
+__host__ __device__ constexpr int coprime_part(int n) {
+  int p = 1;
+  for (int f : {2, 3, 5}) {
+    int q = 1, m = n;
+    for (; m % f == 0; m /= f) q *= f;
+    if (q > 1 && q < n) {
+      p = q;
+      break;
+    }
+  }
+  return p;   // 1: n is a prime power
+}
+__host__ __device__ constexpr int pick_radix(int n) { return n % 4 == 0 ? 4 : (n % 3 == 0 ? 3 : (n % 5 == 0 ? 5 : 2)); }
+__host__ __device__ constexpr int inv_mod(int a, int m) {
+  for (int i = 1; i < m; ++i)
+    if ((a * i) % m == 1) return i;
+  return 1;   // m = 1
 }
 
-// Mixed-radix decimation in time: X[k + M s] = sum_r W_R^{rs} (W_N^{rk} Y_r[k]),
-// Y_r = DFT_M of x[r::R].
 template <typename T, int N, int S> struct Codelet {
-  static __device__ __forceinline__ void run(cplx<T>* x) {
-    constexpr int R = pick_radix(N);
-    constexpr int M = N / R;
-    if constexpr (M == 1) {
-      Small<T, R, S>::run(x);
-    } else {
+  template <InSet IN = all_in<N>()> static __device__ __forceinline__ void run(cplx<T>* x) {
+    if constexpr (small_radix(N)) {
+      Small<T, N, S>::template run<IN>(x);
+    } else if constexpr (coprime_part(N) > 1) {
+      // x[(Q a + P b) mod N], transformed over b (Q points) for each a, then over a (P points);
+      // output (a', b') is X[(Q qi a' + P pi b') mod N] with Q qi = 1 mod P, P pi = 1 mod Q
+      constexpr int P = coprime_part(N), Q = N / P;
       cplx<T> y[N];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        cplx<T> sub[M];
-#pragma unroll
-        for (int m = 0; m < M; ++m) sub[m] = x[m * R + r];
-        Codelet<T, M, S>::run(sub);
-#pragma unroll
-        for (int k = 0; k < M; ++k) y[r * M + k] = sub[k];
-      }
+      outer<P, Q, IN, 0>(x, y);
+      inner<P, Q, IN, 0>(y, x);
+    } else {
+      // decimation in time: X[k + M s] = sum_r W_R^{rs} (W_N^{rk} Y_r[k]), Y_r = DFT_M of x[r::R]
+      constexpr int R = pick_radix(N), M = N / R;
+      cplx<T> y[N];
+      split<R, M, IN, 0>(x, y);
 #pragma unroll
       for (int k = 0; k < M; ++k) {
         cplx<T> z[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) z[r] = twiddle<T, N, S>(r * k, y[r * M + k]);
-        Small<T, R, S>::run(z);
+        Small<T, R, S>::template run<some<R, M, R, 1, IN>()>(z);
 #pragma unroll
         for (int s = 0; s < R; ++s) x[k + M * s] = z[s];
       }
+    }
+  }
+
+ private:
+  // nonzero set of the sub-transform over m < M of x[(off + m step) mod N]
+  template <int M, int step, int off, InSet IN> static constexpr InSet sub_in() {
+    InSet s = 0;
+    for (int m = 0; m < M; ++m)
+      if ((IN >> ((off + m * step) % N)) & 1) s |= 1ull << m;
+    return s;
+  }
+  // set of the a < A whose sub-transform (M points, step, offset a off) has any nonzero input
+  template <int A, int M, int step, int off, InSet IN> static constexpr InSet some() {
+    InSet s = 0;
+    for (int a = 0; a < A; ++a)
+      for (int m = 0; m < M; ++m)
+        if ((IN >> ((a * off + m * step) % N)) & 1) s |= 1ull << a;
+    return s;
+  }
+  template <int P, int Q, InSet IN, int A> static __device__ __forceinline__ void outer(const cplx<T>* x, cplx<T>* y) {
+    if constexpr (A < P) {
+      constexpr InSet in = sub_in<Q, P, Q * A, IN>();
+      cplx<T> t[Q];
+#pragma unroll
+      for (int b = 0; b < Q; ++b) t[b] = (in >> b) & 1 ? x[(Q * A + P * b) % N] : cplx<T>{0, 0};
+      if constexpr (in != 0) Codelet<T, Q, S>::template run<in>(t);
+#pragma unroll
+      for (int b = 0; b < Q; ++b) y[A * Q + b] = t[b];
+      outer<P, Q, IN, A + 1>(x, y);
+    }
+  }
+  template <int P, int Q, InSet IN, int B> static __device__ __forceinline__ void inner(const cplx<T>* y, cplx<T>* x) {
+    if constexpr (B < Q) {
+      constexpr InSet in = some<P, Q, P, Q, IN>();
+      cplx<T> t[P];
+#pragma unroll
+      for (int a = 0; a < P; ++a) t[a] = y[a * Q + B];
+      Codelet<T, P, S>::template run<in>(t);
+#pragma unroll
+      for (int a = 0; a < P; ++a) x[(Q * inv_mod(Q, P) * a + P * inv_mod(P, Q) * B) % N] = t[a];
+      inner<P, Q, IN, B + 1>(y, x);
+    }
+  }
+  template <int R, int M, InSet IN, int A> static __device__ __forceinline__ void split(const cplx<T>* x, cplx<T>* y) {
+    if constexpr (A < R) {
+      constexpr InSet in = sub_in<M, R, A, IN>();
+      cplx<T> t[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m) t[m] = (in >> m) & 1 ? x[m * R + A] : cplx<T>{0, 0};
+      if constexpr (in != 0) Codelet<T, M, S>::template run<in>(t);
+#pragma unroll
+      for (int m = 0; m < M; ++m) y[A * M + m] = t[m];
+      split<R, M, IN, A + 1>(x, y);
     }
   }
 };

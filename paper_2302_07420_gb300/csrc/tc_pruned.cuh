@@ -31,6 +31,12 @@ template <int N, int L> struct Sup {
   static __host__ __device__ constexpr int mil(int c) {
     return (L == N) ? (c <= (N - 1) / 2 ? c : c - N) : (c < H ? c : c - L);
   }
+  // box indices on the support (the nonzero inputs of an inverse pencil)
+  static __host__ __device__ constexpr InSet on() {
+    InSet m = 0;
+    for (int c = 0; c < L; ++c) m |= 1ull << box(c);
+    return m;
+  }
   // compact index of the negated Miller integer (L < N: the support is symmetric and clear of the
   // Nyquist index, so -m is again on the support)
   static __host__ __device__ constexpr int refl(int c) { return c == 0 ? 0 : L - c; }
@@ -83,7 +89,7 @@ __device__ __forceinline__ void pinv_23(cplx<T>* B, Spec spec) {
     for (int i = 0; i < N; ++i) v[i] = cplx<T>{0, 0};
 #pragma unroll
     for (int c2 = 0; c2 < L; ++c2) v[S::box(c2)] = spec(c1, c2, c3);
-    Codelet<T, N, +1>::run(v);
+    Codelet<T, N, +1>::template run<S::on()>(v);
 #pragma unroll
     for (int i2 = 0; i2 < N; ++i2) B[S::bidx(c1, i2, c3)] = v[i2];
   }
@@ -95,7 +101,7 @@ __device__ __forceinline__ void pinv_23(cplx<T>* B, Spec spec) {
     for (int i = 0; i < N; ++i) v[i] = cplx<T>{0, 0};
 #pragma unroll
     for (int c3 = 0; c3 < L; ++c3) v[S::box(c3)] = B[S::bidx(c1, i2, c3)];
-    Codelet<T, N, +1>::run(v);
+    Codelet<T, N, +1>::template run<S::on()>(v);
 #pragma unroll
     for (int i3 = 0; i3 < N; ++i3) B[S::bidx(c1, i2, i3)] = v[i3];
   }
@@ -117,7 +123,7 @@ __device__ __forceinline__ void pass_axis1(cplx<T>* B, Load load, Body body, boo
       for (int i = 0; i < N; ++i) v[i] = cplx<T>{0, 0};
 #pragma unroll
       for (int c1 = 0; c1 < L; ++c1) v[S::box(c1)] = B[S::bidx(c1, i2, i3)];
-      Codelet<T, N, +1>::run(v);
+      Codelet<T, N, +1>::template run<S::on()>(v);
     } else {
 #pragma unroll
       for (int i = 0; i < N; ++i) v[i] = load(i, i2, i3);
