@@ -14,7 +14,8 @@
 //                  3a4 (Alg. 6), 3b3 (Alg. 9), 3b5 (Alg. 11), 3b6 (Alg. 12) fused into one
 //                  FFT chain per (j, q) pair
 //   k_pair_3b4     second pass for 3b4 (Alg. 10), which needs the complete w_j
-//   k_finalize     local terms, 3b6 corrections (Eqs. 3b6_div_scf1/2/3), FFT, box -> sphere
+//   k_local        local terms and 3b6 corrections (Eqs. 3b6_div_scf1/2/3; scalars: k_corr_scalars)
+//   k_finalize     FFT, box -> sphere
 #pragma once
 #include "tc_kernels.cuh"
 
@@ -208,10 +209,8 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
   const cplx<T>* a;
   const cplx<T>* b = nullptr;
   cplx<T>* dst;
-  if (which == 0) {          // n~
-    a = S.n; dst = S.nt;
-  } else if (which == 1) {   // m~_c
-    a = S.m + (size_t)c * G::nn; dst = S.mt + (size_t)c * G::nn;
+  if (which == 0) {          // n~ (block 0) and m~_c (blocks 1 .. 3): n and m, nt and mt are contiguous
+    a = S.n + (size_t)c * G::nn; dst = S.nt + (size_t)c * G::nn;
   } else if (which == 2) {   // FT[h1_c n]  (Alg. 7)
     a = S.h1 + (size_t)c * G::nn; b = S.n; dst = S.spec + (size_t)c * G::nn;
   } else {                   // FT[h5_c]    (Alg. 8)
@@ -228,19 +227,25 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
 
 // Hartree-type convolutions (Delta = 0, G = 0 dropped), blockIdx.y = side.
 //   kind 0: v_H = FT^{-1}[Vh n~]
-//   kind 1: h1_c = FT^{-1}[i G_c u~h n~]                 (c = blockIdx.x)
+//   kind 1: h1_c = FT^{-1}[i G_c u~h n~]
 //   kind 2: v_b2 = FT^{-1}[-i G u~h . m~]
 //   kind 3: t3b1 = FT^{-1}[-i G u~h . FT[h1 n]]         (spectrum in S.spec)
 //   kind 4: t3b2 = FT^{-1}[-i G u~h . FT[h5]]           (spectrum in S.spec)
-//   kind 5: vu_s = FT^{-1}[u~_s n~] (no 1/Omega)        (s = blockIdx.x)
+//   kind 5: vu_s = FT^{-1}[u~_s n~] (no 1/Omega)
+// The kinds that need n~ and m~ only (0, 1, 2 and 5) run as the 7 blocks of one launch (kind_or_all = -1): a
+// launch of one CTA per field is one FFT's latency whatever its block count (hartree stage of the
+// 14-electron gas, FP64 16^3: 0.42 ms in nine launches, 0.25 in five).
 template <typename T, int N>
 __global__ void __launch_bounds__(Cfg<N>::threads)
-    k_hartree_inv(Params<T> P, int kind) {
+    k_hartree_inv(Params<T> P, int kind_or_all) {
   using G = Geo<N>;
   extern __shared__ __align__(16) unsigned char smraw[];
   cplx<T>* V = work_vol<T, N>(smraw, P.scratch);
   const SideArgs<T>& S = P.side[blockIdx.y];
-  const int c = blockIdx.x;
+  // kind_or_all < 0: blocks 0 | 1-3 | 4 | 5-6 = kinds 0 | 1 | 2 | 5
+  const int bx = blockIdx.x;
+  const int kind = kind_or_all >= 0 ? kind_or_all : bx == 0 ? 0 : bx < 4 ? 1 : bx == 4 ? 2 : 5;
+  const int c = kind_or_all >= 0 ? bx : kind == 1 ? bx - 1 : kind == 5 ? bx - 5 : 0;
   const T zero3[3] = {0, 0, 0};
   const PComp<T> qc = pcomp_setup<T>(P, nullptr, kind == 1 ? c : 0);
   cplx<T>* dst = kind == 0 ? S.vH : kind == 1 ? S.h1 + (size_t)c * G::nn : kind == 2 ? S.vb2 : kind == 3 ? S.t3b1
@@ -847,8 +852,78 @@ __global__ void __launch_bounds__(Cfg<N>::threads, 1) k_pair_3b4(Params<T> P) {
 }
 
 // ---------------------------------------------------------------------------
-// Finalize: acc += vloc ket_j + s2b tw2bh1 h1 . grad ket_j + tw3a3 h1 . w_j + 3b6 corrections,
-// then out(G) = FT[acc](G) on the sphere of k_j (FP64 interleaved complex).
+// Scalars of the 3b6 corrections of every (output, occupied mu at its k): in place of the six sums
+// in cs, alpha = (f_mu / Omega^2) (c n0 O + a_pp X_pp + a_ap X_ap) and omega = (f_mu / Omega^2) O in
+// the compute precision (4 values of T at the start of the entry), so that k_local evaluates
+// sum_mu ket_mu (alpha + omega v(r)), v = a_pp vu_pp + a_ap vu_ap, without FP64 work per grid point.
+template <typename T, int N> __global__ void k_corr_scalars(Params<T> P) {
+  const SideArgs<T>& S = P.side[blockIdx.y];
+  const int nit = P.sym ? P.nirr * P.nb : P.nj_out;
+  const double a0 = 4.0 * 3.14159265358979323846 * P.A[0] / P.Nk, a1 = 4.0 * 3.14159265358979323846 * P.A[1] / P.Nk;
+  const double n0x = (double)S.nt[0].x, n0y = (double)S.nt[0].y, cc = P.corr_c[0] + P.corr_c[1];
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nit * P.no; e += gridDim.x * blockDim.x) {
+    const int item = e / P.no, mu = e % P.no;
+    const int jo = P.sym ? P.irr[item / P.nb] * P.nb + item % P.nb : item;
+    double* cs = S.cs + ((size_t)jo * P.no + mu) * 6;
+    const double f = P.occ[(P.j0 + jo) / P.nb * P.nb + mu], fq = f * P.invOm2;
+    cplx<T>* o = reinterpret_cast<cplx<T>*>(cs);
+    if ((T)(f / P.Nk) == T(0)) {   // the chains skip such a partner: its sums are unwritten
+      o[0] = o[1] = cplx<T>{0, 0};
+      continue;
+    }
+    const double ox = cs[0], oy = cs[1], x0 = cs[2], y0 = cs[3], x1 = cs[4], y1 = cs[5];
+    const double ax = fq * (cc * (n0x * ox - n0y * oy) + a0 * x0 + a1 * x1);
+    const double ay = fq * (cc * (n0x * oy + n0y * ox) + a0 * y0 + a1 * y1);
+    o[0] = cplx<T>{(T)ax, (T)ay};
+    o[1] = cplx<T>{(T)(fq * ox), (T)(fq * oy)};
+  }
+}
+
+// Local terms of every output, one thread per grid point and output:
+//   acc += vloc ket_j + s2b tw2bh1 h1 . grad ket_j + tw3a3 h1 . w_j + 3b6 corrections.
+// Bound by the loads of acc, w and grad ket (9 volumes per output).  It used to be the load of
+// k_finalize's first FFT pass, whose one CTA per output walked the occupied mu of every grid point with
+// FP64 scalars: 15.8 ms of a 48^3, 57-band apply (337 ms), 0.31 ms of the 14-electron FP64 one (2.7 ms).
+template <typename T, int N> __global__ void __launch_bounds__(256) k_local(Params<T> P) {
+  const SideArgs<T>& S = P.side[blockIdx.z];
+  const size_t NN = (size_t)N * N * N;
+  const int item = blockIdx.x;
+  const int jo = P.sym ? P.irr[item / P.nb] * P.nb + item % P.nb : item;
+  const int j = P.j0 + jo, kj = j / P.nb;
+  const T t2bh1 = P.tw[T2BH1] * S.s2b, t3a3 = P.tw[T3A3], t3b6 = P.tw[T3B6];
+  const bool corr = P.div && t3b6 != T(0) && !P.band;
+  const T a0 = (T)(4.0 * 3.14159265358979323846 * P.A[0] / P.Nk), a1 = (T)(4.0 * 3.14159265358979323846 * P.A[1] / P.Nk);
+  const cplx<T>* ketj = S.ket + (size_t)j * NN;
+  const cplx<T>* gketj = S.gket + (size_t)j * 3 * NN;
+  const cplx<T>* w = S.w + (size_t)jo * 3 * NN;
+  cplx<T>* acc = S.acc + (size_t)jo * NN;
+  for (int g = blockIdx.y * blockDim.x + threadIdx.x; g < (int)NN; g += gridDim.y * blockDim.x) {
+    cplx<T> v = acc[g] + S.vloc[g] * ketj[g];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const cplx<T> h = S.h1[d * NN + g];
+      v = v + t2bh1 * (h * gketj[d * NN + g]) + t3a3 * (h * w[d * NN + g]);
+    }
+    if (corr) {
+      // sum_q f_q ket_q (1/Omega^2) sum_s [c_s n0 O_qj + (4 pi A_s/Nk)(O_qj vu_s + X_s)]
+      const cplx<T> vu = a0 * S.vu[g] + a1 * S.vu[NN + g];
+      const cplx<T>* ket = S.ket + (size_t)kj * P.nb * NN + g;
+      cplx<T> s = {0, 0};
+#pragma unroll 4
+      for (int mu = 0; mu < P.no; ++mu) {
+        const cplx<T>* cs = reinterpret_cast<const cplx<T>*>(S.cs + ((size_t)jo * P.no + mu) * 6);
+        const cplx<T> al = cs[0], om = cs[1];
+        if (al.x == T(0) && al.y == T(0) && om.x == T(0) && om.y == T(0)) continue;
+        s = s + ket[(size_t)mu * NN] * (al + om * vu);
+      }
+      v = v + t3b6 * s;
+    }
+    acc[g] = v;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Finalize: out(G) = FT[acc](G) on the sphere of k_j (FP64 interleaved complex).
 template <typename T, int N>
 __global__ void __launch_bounds__(Cfg<N>::threads)
     k_finalize(Params<T> P, double2* outR, double2* outL, const int* __restrict__ box_index) {
@@ -860,47 +935,10 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
   double2* out = side == 0 ? outR : outL;
   if (out == nullptr) return;
   const int jo = P.sym ? P.irr[blockIdx.x / P.nb] * P.nb + blockIdx.x % P.nb : blockIdx.x;
-  const int j = P.j0 + jo, kj = j / P.nb;
-  const size_t NN = G::nn;
-  const cplx<T>* ketj = S.ket + (size_t)j * NN;
-  const cplx<T>* gketj = S.gket + (size_t)j * 3 * NN;
-  const cplx<T>* acc = S.acc + (size_t)jo * NN;
-  const cplx<T>* w = S.w + (size_t)jo * 3 * NN;
-  const T t2bh1 = P.tw[T2BH1] * S.s2b, t3a3 = P.tw[T3A3];
-  const bool corr = P.div && P.tw[T3B6] != T(0) && !P.band;
-  const T a0 = (T)(4.0 * 3.14159265358979323846 * P.A[0] / P.Nk), a1 = (T)(4.0 * 3.14159265358979323846 * P.A[1] / P.Nk);
-  const double n0x = corr ? (double)S.nt[0].x : 0.0, n0y = corr ? (double)S.nt[0].y : 0.0;
-  fwd3d<T, N>(
-      V,
-      [&](int a, int b, int c) {
-        const int g = G::gidx(a, b, c);
-        const cplx<T> kv = ketj[g];
-        cplx<T> v = acc[g] + S.vloc[g] * kv;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          const cplx<T> h = S.h1[d * NN + g];
-          v = v + t2bh1 * (h * gketj[d * NN + g]) + t3a3 * (h * w[d * NN + g]);
-        }
-        if (corr) {
-          // sum_q f_q ket_q (1/Omega^2) sum_s [c_s n0 O_qj + (4 pi A_s/Nk)(O_qj vu_s + X_s)]
-          cplx<T> s = {0, 0};
-          for (int mu = 0; mu < P.no; ++mu) {
-            const int q = kj * P.nb + mu;
-            const double fq = P.occ[q];
-            if (fq == 0.0) continue;
-            const double* cs = S.cs + ((size_t)jo * P.no + mu) * 6;
-            const cplx<T> O = {(T)cs[0], (T)cs[1]};
-            const cplx<T> X0 = {(T)cs[2], (T)cs[3]}, X1 = {(T)cs[4], (T)cs[5]};
-            const double cc = P.corr_c[0] + P.corr_c[1];
-            const cplx<T> cn = {(T)(cc * n0x), (T)(cc * n0y)};
-            cplx<T> t = cn * O + a0 * (O * S.vu[g] + X0) + a1 * (O * S.vu[NN + g] + X1);
-            s = s + (T)(fq * P.invOm2) * (S.ket[(size_t)q * NN + g] * t);
-          }
-          v = v + P.tw[T3B6] * s;
-        }
-        return v;
-      },
-      [&](int a, int b, int c, cplx<T> v) { V[G::sidx(a, b, c)] = P.invN * v; });
+  const int kj = (P.j0 + jo) / P.nb;
+  const cplx<T>* acc = S.acc + (size_t)jo * G::nn;
+  fwd3d<T, N>(V, [&](int a, int b, int c) { return ldg(acc + G::gidx(a, b, c)); },
+              [&](int a, int b, int c, cplx<T> v) { V[G::sidx(a, b, c)] = P.invN * v; });
   __syncthreads();
   double2* o = out + (size_t)jo * P.npw_max;
   for (int g = threadIdx.x; g < P.npw_max; g += blockDim.x) {

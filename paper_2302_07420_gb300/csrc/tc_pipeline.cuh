@@ -288,7 +288,7 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   // band points: every divergence correction (all need div_correction) and the fields they take
   const bool band_corr = band && P.div;
   const int pw_blocks = 2 * 152;
-  int nl[6] = {1, 9, 0, 1, 1, 1};   // kernel launches per stage
+  int nl[6] = {1, 5, 0, 1, 1, 2};   // kernel launches per stage
   // pair densities whose spectra fit the compiled support take the pruned transforms
   constexpr int LP = kPruneL<N>;
   const bool pruned = LP < N && ctx->pair_support <= LP;
@@ -348,13 +348,17 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   stage_mark(ctx, st, 1);
   k_density<T, N><<<dim3(pw_blocks, nsides), 256, 0, st>>>(P);
   TC_CHECK_LAUNCH("k_density");
-  k_spec_fwd<T, N><<<dim3(1, nsides), TH, vb1, st>>>(P, 0);
-  k_spec_fwd<T, N><<<dim3(3, nsides), TH, vb1, st>>>(P, 1);
+  k_spec_fwd<T, N><<<dim3(4, nsides), TH, vb1, st>>>(P, 0);
   TC_CHECK_LAUNCH("k_spec_fwd");
-  k_hartree_inv<T, N><<<dim3(1, nsides), TH, vb1, st>>>(P, 0);
-  k_hartree_inv<T, N><<<dim3(3, nsides), TH, vb1, st>>>(P, 1);
-  k_hartree_inv<T, N><<<dim3(1, nsides), TH, vb1, st>>>(P, 2);
-  k_hartree_inv<T, N><<<dim3(2, nsides), TH, vb1, st>>>(P, 5);
+  if (Fit<T, N>::one || ctx->scratch_bytes >= (size_t)7 * nsides * vb) {
+    k_hartree_inv<T, N><<<dim3(7, nsides), TH, vb1, st>>>(P, -1);
+  } else {   // a scratch for fewer work volumes than that (a single orbital): one kind at a time
+    k_hartree_inv<T, N><<<dim3(1, nsides), TH, vb1, st>>>(P, 0);
+    k_hartree_inv<T, N><<<dim3(3, nsides), TH, vb1, st>>>(P, 1);
+    k_hartree_inv<T, N><<<dim3(1, nsides), TH, vb1, st>>>(P, 2);
+    k_hartree_inv<T, N><<<dim3(2, nsides), TH, vb1, st>>>(P, 5);
+    nl[1] += 3;
+  }
   TC_CHECK_LAUNCH("k_hartree_inv");
   k_spec_fwd<T, N><<<dim3(3, nsides), TH, vb1, st>>>(P, 2);
   k_hartree_inv<T, N><<<dim3(1, nsides), TH, vb1, st>>>(P, 3);
@@ -523,6 +527,12 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
     TC_CHECK_LAUNCH("k_band_corr");
     nl[5] += 1;
   }
+  if (P.div && tw[T3B6] != 0 && !P.band) {
+    k_corr_scalars<T, N><<<dim3((nj_items * S.no + 255) / 256, nsides), 256, 0, st>>>(P);
+    nl[5] += 1;
+  }
+  k_local<T, N><<<dim3(nj_items, (S.N + 255) / 256, nsides), 256, 0, st>>>(P);
+  TC_CHECK_LAUNCH("k_local");
   k_finalize<T, N><<<dim3(nj_items, nsides), TH, vb1, st>>>(P, outR, outL, ctx->d_box_index);
   TC_CHECK_LAUNCH("k_finalize");
   if (P.sym && P.nirr < S.Nk) {
