@@ -96,7 +96,7 @@ template <typename T> void* upload_as(const std::vector<double>& v, cudaError_t&
 void free_all(tc_ctx* c) {
   void* ptrs[] = {c->d_box_index, c->d_kpg, c->d_delta_id, c->d_delta, c->d_tabV, c->d_tabU, c->d_hartV,
                   c->d_hartU, c->d_hartUs, c->d_occ, c->ws_owned ? c->d_ws : nullptr, c->d_in_phi, c->d_in_chi,
-                  c->d_out_R, c->d_out_L, c->d_edot, c->d_npw, c->d_status, c->d_band, c->d_bs, c->d_kd64,
+                  c->d_out_R, c->d_out_L, c->d_edot, c->d_npw, c->d_status, c->d_band, c->d_bs, c->d_kd64, c->d_norms,
                   c->d_mirror};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -515,6 +515,8 @@ int init_context(const tc_params* params, bool own_workspace, tc_ctx** out, std:
   if (e == cudaSuccess) ok(cudaMalloc((void**)&c->d_edot, nj * sizeof(double2)));
   if (e == cudaSuccess) ok(cudaMalloc((void**)&c->d_npw, S.npw.size() * sizeof(int)));
   if (e == cudaSuccess) ok(cudaMemcpy(c->d_npw, S.npw.data(), S.npw.size() * sizeof(int), cudaMemcpyHostToDevice));
+  if (e == cudaSuccess && c->prec == TC_FP64)   // 16-byte entries (tc::Norm)
+    ok(cudaMalloc((void**)&c->d_norms, 16 * (2 * nj_all + 2 * norms_per_side(c->nj_out, S.Nk, S.no))));
   if (e == cudaSuccess) ok(cudaMalloc((void**)&c->d_status, sizeof(int)));
   if (e == cudaSuccess) ok(cudaMallocHost((void**)&c->h_status, sizeof(int)));
   if (e == cudaSuccess) ok(cudaMallocHost((void**)&c->h_edot, nj * sizeof(double2)));

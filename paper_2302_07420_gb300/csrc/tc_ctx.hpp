@@ -9,6 +9,7 @@
 
 namespace tc {
 struct BatchState;
+struct Norm;
 struct DavState;
 // Offsets of the workspace pieces of one context inside its workspace block.
 struct WsLayout {
@@ -87,6 +88,8 @@ struct tc_ctx {
   // quarter of the free device memory, else null (each side computes its own)
   void* d_mirror = nullptr;
   size_t mirror_bytes = 0;
+  // FP64: norms of the real-space fields (fixed-point transforms); null: in dead base fields
+  tc::Norm* d_norms = nullptr;
   // cluster-distributed pair kernels that can be scheduled on this device (bit 0 chain, 1 3b4,
   // 2 occupied pairs; tc_cluster.cuh), set by prepare_kernels
   int cluster_ok = 0;
@@ -136,6 +139,8 @@ WsLayout ws_layout(const tc_ctx* c);
 void choose_splits(tc_ctx* c);
 // n^3 volumes of one side's field block (see fill_side).
 size_t side_field_vols(int Nk, int nb, int no, int so_max, int sc_max, int nj_out, int nkb, int so_band);
+// Norms of one side: n, Y, h3b, w (see fill_side).
+inline size_t norms_per_side(int nj_out, int Nk, int no) { return 1 + (size_t)6 * nj_out + (size_t)3 * Nk * no; }
 void ws_assign(tc_ctx* c, char* base, const WsLayout& L);
 // Both operator sides into outR / outL (device pointers) on st, all terms of term_mask.
 int apply_device(tc_ctx* c, const double2* phi, const double2* chi, double2* outR, double2* outL, cudaStream_t st);

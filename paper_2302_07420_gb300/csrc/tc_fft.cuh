@@ -64,6 +64,7 @@ constexpr int kTwTotal = tw_offset(48) + 48;
 // uploads its own copy in prepare_kernels.
 static __constant__ double c_tw64[2 * kTwTotal];
 static __constant__ float c_tw32[2 * kTwTotal];
+static __constant__ long long c_twfx[2 * kTwTotal];   // 2^63 w, for the fixed-point transforms
 
 template <typename T> __device__ __forceinline__ cplx<T> tw_load(int idx);
 template <> __device__ __forceinline__ cplx<double> tw_load<double>(int idx) { return {c_tw64[2 * idx], c_tw64[2 * idx + 1]}; }
@@ -78,9 +79,15 @@ template <typename T, int N, int S> __device__ __forceinline__ cplx<T> twiddle(i
     if (q == 2) return cplx<T>{-v.x, -v.y};
     return (q == 1) ? mul_si<T, S>(v) : mul_si<T, -S>(v);
   }
-  cplx<T> w = tw_load<T>(tw_offset(N) + e);   // exp(-2 pi i e/N)
-  if (S > 0) w.y = -w.y;
-  return v * w;
+  if constexpr (T(0.5) == T(0)) {
+    const int i = tw_offset(N) + e;
+    const long long wr = c_twfx[2 * i], wi = S > 0 ? -c_twfx[2 * i + 1] : c_twfx[2 * i + 1];
+    return {(__mul64hi(v.x, wr) - __mul64hi(v.y, wi)) << 1, (__mul64hi(v.x, wi) + __mul64hi(v.y, wr)) << 1};
+  } else {
+    cplx<T> w = tw_load<T>(tw_offset(N) + e);   // exp(-2 pi i e/N)
+    if (S > 0) w.y = -w.y;
+    return v * w;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -107,18 +114,89 @@ __device__ __forceinline__ cplx<float> operator-(cplx<float> a, cplx<float> b) {
   const float2 r = __ffma2_rn(make_float2(b.x, b.y), make_float2(-1.f, -1.f), make_float2(a.x, a.y));
   return {r.x, r.y};
 }
-// a + s b, s real
-template <typename T> __device__ __forceinline__ cplx<T> axpy(T s, cplx<T> b, cplx<T> a) {
+// Transforms run in float, double or in 64-bit fixed point (T = long long, told by T(0.5) == 0; its
+// scaling is in tc_fixed.cuh).
+// Real factors K of the butterflies, by name: 1/2, sqrt(3)/2, sqrt(1/2), cos(2 pi/5), -cos(4 pi/5),
+// sin(2 pi/5), sin(4 pi/5)/sin(2 pi/5); floating and as round(K 2^64) for the fixed-point transforms.
+enum { KH, KS3, KR8, KC1, KC2, KS1, KRHO };
+__host__ __device__ constexpr double kval(int k) {
+  constexpr double v[] = {0.5,
+                          0.86602540378443864676372317075294,
+                          0.70710678118654752440084436210485,
+                          0.30901699437494742410229341718282,
+                          0.80901699437494742410229341718282,
+                          0.95105651629515357211643933337938,
+                          0.61803398874989484820458683436564};
+  return v[k];
+}
+__host__ __device__ constexpr unsigned long long kfix(int k) {
+  constexpr unsigned long long v[] = {0x8000000000000000ull, 0xddb3d742c265539eull, 0xb504f333f9de6484ull,
+                                      0x4f1bbcdcbfa53e0bull, 0xcf1bbcdcbfa53e0bull, 0xf378709a22a7faf3ull,
+                                      0x9e3779b97f4a7c16ull};
+  return v[k];
+}
+// x K in fixed point, rounded down: the high word of the signed product; a K above 1/2 reads as K - 1 there
+template <int K> __device__ __forceinline__ long long fxmul(long long x) {
+  if constexpr (K == KH) return x >> 1;
+  else if constexpr ((kfix(K) >> 63) == 0) return __mul64hi(x, (long long)kfix(K));
+  else return __mul64hi(x, (long long)kfix(K)) + x;
+}
+// s K b
+template <int K, int SG, typename T> __device__ __forceinline__ cplx<T> scalek(cplx<T> b) {
+  if constexpr (sizeof(cplx<T>) == 16 && T(0.5) == T(0)) {
+    const cplx<T> m = {fxmul<K>(b.x), fxmul<K>(b.y)};
+    return SG > 0 ? m : cplx<T>{-m.x, -m.y};
+  } else {
+    constexpr T s = T(SG * kval(K));
+    return {s * b.x, s * b.y};
+  }
+}
+// a + s K b
+template <int K, int SG, typename T> __device__ __forceinline__ cplx<T> axpy(cplx<T> b, cplx<T> a) {
   if constexpr (sizeof(T) == 4) {
+    constexpr float s = float(SG * kval(K));
     const float2 r = __ffma2_rn(make_float2(b.x, b.y), make_float2(s, s), make_float2(a.x, a.y));
     return {r.x, r.y};
+  } else if constexpr (T(0.5) == T(0)) {
+    const cplx<T> m = {fxmul<K>(b.x), fxmul<K>(b.y)};
+    return SG > 0 ? cplx<T>{a.x + m.x, a.y + m.y} : cplx<T>{a.x - m.x, a.y - m.y};
   } else {
+    constexpr T s = T(SG * kval(K));
     return {fma(s, b.x, a.x), fma(s, b.y, a.y)};
   }
 }
-// a + s i b, s real
-template <typename T> __device__ __forceinline__ cplx<T> axpy_i(T s, cplx<T> b, cplx<T> a) {
-  return {fma(-s, b.y, a.x), fma(s, b.x, a.y)};
+// a + s K i b
+template <int K, int SG, typename T> __device__ __forceinline__ cplx<T> axpy_i(cplx<T> b, cplx<T> a) {
+  if constexpr (T(0.5) == T(0)) {
+    const cplx<T> m = {fxmul<K>(b.x), fxmul<K>(b.y)};
+    return SG > 0 ? cplx<T>{a.x - m.y, a.y + m.x} : cplx<T>{a.x + m.y, a.y - m.x};
+  } else {
+    constexpr T s = T(SG * kval(K));
+    return {fma(-s, b.y, a.x), fma(s, b.x, a.y)};
+  }
+}
+// p = a + K b, m = a - K b (one product in fixed point)
+template <int K, typename T> __device__ __forceinline__ void both(cplx<T> b, cplx<T> a, cplx<T>& p, cplx<T>& m) {
+  if constexpr (T(0.5) == T(0)) {
+    const cplx<T> t = {fxmul<K>(b.x), fxmul<K>(b.y)};
+    p = {a.x + t.x, a.y + t.y};
+    m = {a.x - t.x, a.y - t.y};
+  } else {
+    p = axpy<K, 1>(b, a);
+    m = axpy<K, -1>(b, a);
+  }
+}
+// p = a + S K i b, m = a - S K i b
+template <int K, int S, typename T> __device__ __forceinline__ void rot2(cplx<T> b, cplx<T> a, cplx<T>& p, cplx<T>& m) {
+  if constexpr (T(0.5) == T(0)) {
+    const cplx<T> t = {fxmul<K>(b.x), fxmul<K>(b.y)};
+    const cplx<T> u = {a.x - t.y, a.y + t.x}, v = {a.x + t.y, a.y - t.x};
+    p = S > 0 ? u : v;
+    m = S > 0 ? v : u;
+  } else {
+    p = axpy_i<K, S>(b, a);
+    m = axpy_i<K, -S>(b, a);
+  }
 }
 // sum and difference of values that may be known zeros
 template <bool ZA, bool ZB, typename T> __device__ __forceinline__ cplx<T> addz(cplx<T> a, cplx<T> b) {
@@ -151,17 +229,17 @@ template <typename T, int S> struct Small<T, 2, S> {
 template <typename T, int S> struct Small<T, 3, S> {
   template <InSet IN> static __device__ __forceinline__ void run(cplx<T>* z) {
     constexpr bool A = IN & 1, B = IN & 2, C = IN & 4;
-    const T h = T(0.5), s3 = T(S * 0.86602540378443864676372317075294);   // sqrt(3)/2
     const cplx<T> a = z[0];
     if constexpr (!B && !C) {
       z[1] = a;
       z[2] = a;
     } else {
       const cplx<T> t1 = addz<B, C>(z[1], z[2]), t2 = subz<B, C>(z[1], z[2]);
-      const cplx<T> m = A ? axpy<T>(-h, t1, a) : cplx<T>{-h * t1.x, -h * t1.y};
+      cplx<T> m;
+      if constexpr (A) m = axpy<KH, -1>(t1, a);
+      else m = scalek<KH, -1>(t1);
       z[0] = addz<A, true>(a, t1);
-      z[1] = axpy_i<T>(s3, t2, m);
-      z[2] = axpy_i<T>(-s3, t2, m);
+      rot2<KS3, S>(t2, m, z[1], z[2]);
     }
   }
 };
@@ -186,9 +264,6 @@ template <typename T, int S> struct Small<T, 4, S> {
 template <typename T, int S> struct Small<T, 5, S> {
   template <InSet IN> static __device__ __forceinline__ void run(cplx<T>* z) {
     constexpr bool A = IN & 1, B1 = IN & 2, B2 = IN & 4, B3 = IN & 8, B4 = IN & 16, P = B1 || B4, Q = B2 || B3;
-    // cos(2 pi/5), cos(4 pi/5), sin(2 pi/5), sin(4 pi/5)/sin(2 pi/5)
-    const T c1 = T(0.30901699437494742410229341718282), c2 = T(-0.80901699437494742410229341718282);
-    const T s1 = T(S * 0.95105651629515357211643933337938), r = T(0.61803398874989484820458683436564);
     const cplx<T> x0 = A ? z[0] : cplx<T>{0, 0};
     if constexpr (!P && !Q) {
       z[1] = z[2] = z[3] = z[4] = x0;
@@ -197,29 +272,27 @@ template <typename T, int S> struct Small<T, 5, S> {
                     t4 = subz<B2, B3>(z[2], z[3]);
       cplx<T> a1 = x0, a2 = x0, b1, b2;
       if constexpr (P) {
-        a1 = axpy<T>(c1, t1, a1);
-        a2 = axpy<T>(c2, t1, a2);
+        a1 = axpy<KC1, 1>(t1, a1);
+        a2 = axpy<KC2, -1>(t1, a2);
       }
       if constexpr (Q) {
-        a1 = axpy<T>(c2, t2, a1);
-        a2 = axpy<T>(c1, t2, a2);
+        a1 = axpy<KC2, -1>(t2, a1);
+        a2 = axpy<KC1, 1>(t2, a2);
       }
       // sin parts over sin(2 pi/5): t3 + r t4 and r t3 - t4
       if constexpr (P && Q) {
-        b1 = axpy<T>(r, t4, t3);
-        b2 = axpy<T>(r, t3, cplx<T>{-t4.x, -t4.y});
+        b1 = axpy<KRHO, 1>(t4, t3);
+        b2 = axpy<KRHO, 1>(t3, cplx<T>{-t4.x, -t4.y});
       } else if constexpr (P) {
         b1 = t3;
-        b2 = cplx<T>{r * t3.x, r * t3.y};
+        b2 = scalek<KRHO, 1>(t3);
       } else {
-        b1 = cplx<T>{r * t4.x, r * t4.y};
+        b1 = scalek<KRHO, 1>(t4);
         b2 = cplx<T>{-t4.x, -t4.y};
       }
       z[0] = addz<A, true>(x0, addz<P, Q>(t1, t2));
-      z[1] = axpy_i<T>(s1, b1, a1);
-      z[4] = axpy_i<T>(-s1, b1, a1);
-      z[2] = axpy_i<T>(s1, b2, a2);
-      z[3] = axpy_i<T>(-s1, b2, a2);
+      rot2<KS1, S>(b1, a1, z[1], z[4]);
+      rot2<KS1, S>(b2, a2, z[2], z[3]);
     }
   }
 };
@@ -228,7 +301,6 @@ template <typename T, int S> struct Small<T, 8, S> {
   template <InSet IN> static __device__ __forceinline__ void run(cplx<T>* z) {
     constexpr InSet EV = (IN & 1) | ((IN >> 1) & 2) | ((IN >> 2) & 4) | ((IN >> 3) & 8);
     constexpr InSet OD = ((IN >> 1) & 1) | ((IN >> 2) & 2) | ((IN >> 3) & 4) | ((IN >> 4) & 8);
-    const T r = T(0.70710678118654752440084436210485);
     cplx<T> e[4] = {z[0], z[2], z[4], z[6]}, o[4] = {z[1], z[3], z[5], z[7]};
     if constexpr (EV != 0) Small<T, 4, S>::template run<EV>(e);
     else e[0] = e[1] = e[2] = e[3] = cplx<T>{0, 0};
@@ -246,10 +318,8 @@ template <typename T, int S> struct Small<T, 8, S> {
       // exp(S i pi/4) o = r u1 and exp(S 3 i pi/4) o = -r u3
       const cplx<T> u1 = S > 0 ? cplx<T>{o[1].x - o[1].y, o[1].y + o[1].x} : cplx<T>{o[1].x + o[1].y, o[1].y - o[1].x};
       const cplx<T> u3 = S > 0 ? cplx<T>{o[3].x + o[3].y, o[3].y - o[3].x} : cplx<T>{o[3].x - o[3].y, o[3].y + o[3].x};
-      z[1] = axpy<T>(r, u1, e[1]);
-      z[5] = axpy<T>(-r, u1, e[1]);
-      z[3] = axpy<T>(-r, u3, e[3]);
-      z[7] = axpy<T>(r, u3, e[3]);
+      both<KR8>(u1, e[1], z[1], z[5]);
+      both<KR8>(u3, e[3], z[7], z[3]);
     }
   }
 };

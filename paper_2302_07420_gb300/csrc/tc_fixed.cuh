@@ -1,0 +1,257 @@
+// 64-bit fixed-point transforms for the FP64 pair kernels.
+//
+// The FP64 pipe of GB300 gives 1.6 additions or fused multiply-adds per clock and SM, the integer
+// pipe 57 64-bit additions and 5.8 64-bit high products (measured, 1024 threads): a 24-point codelet
+// (252 operations, 28 of them products by constants) takes 157 clocks per thread and SM in FP64
+// and about 11 in integers.  So the work volumes of the FP64 pruned kernels hold integers
+// v 2^(62 - e), with one exponent e per transform and pass; the products in real space, the spectral
+// multiplications and every accumulator stay in FP64, and FP32 kernels use none of this.
+//
+// Scaling.  An integer transform neither overflows nor loses bits when e follows from a bound: with
+// |v| <= b0 for every nonzero input and sum |v| <= bt, every partial sum of the first, second and
+// third pass over len values is at most b_k = min(len^k b0, bt), and every intermediate of a codelet
+// is a combination of its inputs with weights of modulus at most 1, taken apart into x +- y at most
+// once (a factor sqrt(2)).  With e_k = ceil(log2 b_k) the magnitudes stay below sqrt(2) 2^62 < 2^63.
+// Values are converted at e_1 and shifted right, rounded, by e_2 - e_1 and e_3 - e_2 before the second
+// and third pass.  The rounding left in a result is about 1.5 units of 2^(e_3 - 62): bt is a few to
+// some tens of times the result's root mean square, so this lies below the 2^-53 sqrt(log2 N) of an
+// FP64 transform: against 64-bit results the 3x3x3 apply is off by 1.5e-15 (1.8e-15 in FP64
+// arithmetic), and it takes 222 ms instead of 499; the 2x2x2 gradient 151 instead of 324.  Bounds come from the 2- and max norms of the real-space factors (k_norms;
+// |sum a b| <= |a|_2 |b|_2) and, for spectra, from sums of upper-rounded floats over the spectrum.
+// A bound that is not finite (an infinity or NaN among the inputs) poisons the transform: all
+// its results are NaN, as a floating-point transform of such a volume gives.
+#pragma once
+#include "tc_kernels.cuh"
+
+namespace tc {
+
+// Element type of a work volume: fixed point for FP64 kernels.
+template <typename T> struct Work { using type = cplx<T>; };
+template <> struct Work<double> { using type = cplx<long long>; };
+template <typename T> using WorkT = typename Work<T>::type;
+
+// Scale of one transform (empty in FP32).
+template <typename T> struct Scale {};
+template <> struct Scale<double> {
+  int k_in;        // inputs are converted as v 2^k_in
+  int s2, s3;      // right shifts before the second and third pass
+  int hi_out;      // exponent field added to results (e_3 - 62, shifted into the high word)
+  int poison;      // bits set in the high word of every result: NaN when a bound is not finite
+};
+
+// Smallest e with b < 2^e (b >= 0), clamped to where every shifted exponent below stays normal.
+__device__ __forceinline__ int fx_exp(double b) {
+  const int e = ((__double2hiint(b) >> 20) & 0x7ff) - 1022;
+  return e < -400 ? -400 : e;
+}
+constexpr int ceil_log2(long long v) { return v <= 1 ? 0 : 1 + ceil_log2((v + 1) / 2); }
+
+// Scale of a transform over LEN nonzero values per axis with |v| <= b0 and sum |v| <= bt.
+template <typename T, int LEN> __device__ __forceinline__ Scale<T> fx_scale(double b0, double bt) {
+  Scale<T> s;
+  if constexpr (sizeof(T) == 8) {
+    constexpr int l1 = ceil_log2(LEN), l2 = ceil_log2((long long)LEN * LEN), l3 = ceil_log2((long long)LEN * LEN * LEN);
+    // the norms themselves are rounded: one part in 10^6 on top
+    const int x0 = fx_exp(b0 * 1.000001), xt = fx_exp(bt * 1.000001);
+    const int e3 = min(x0 + l3, xt), e1 = min(x0 + l1, e3), e2 = min(x0 + l2, e3);
+    s.k_in = 62 - e1;
+    s.s2 = e2 - e1;
+    s.s3 = e3 - e2;
+    s.hi_out = (e3 - 62) << 20;
+    s.poison = (xt < 900 && x0 < 900) ? 0 : 0x7ff80000;   // (fx_exp of an infinity or NaN: 1025)
+  }
+  return s;
+}
+
+// v 2^k to the nearest integer, in integer instructions (the conversion instruction runs at the FP64
+// pipe's rate).  |v| 2^k < sqrt(2) 2^62 by the bound, so the shift is not negative; a shift beyond 63
+// (zero among the values) gives 0.
+__device__ __forceinline__ long long to_fx(double v, int k) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  unsigned long long m = ((unsigned long long)((unsigned)(hi & 0xfffff) | 0x100000u) << 32 | (unsigned)lo) << 11;
+  const int t = 1085 - k - ((hi >> 20) & 0x7ff);
+  asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(t));   // twice the magnitude; clamps the shift
+  const long long r = (long long)((m + 1) >> 1), s = (long long)(hi >> 31);
+  return (r ^ s) - s;
+}
+__device__ __forceinline__ cplx<long long> to_work(cplx<double> v, const Scale<double>& s) {
+  return {to_fx(v.x, s.k_in), to_fx(v.y, s.k_in)};
+}
+__device__ __forceinline__ cplx<float> to_work(cplx<float> v, const Scale<float>&) { return v; }
+// v 2^(e_3 - 62), rounded to nearest, in integer instructions
+__device__ __forceinline__ double from_fx(long long v, const Scale<double>& s) {
+  const long long sg = v >> 63;
+  const unsigned long long a = (unsigned long long)((v ^ sg) - sg);
+  const int lz = __clzll((long long)a);
+  unsigned long long m = a << (lz & 63);
+  m = (m >> 11) + ((m >> 10) & 1);                       // 53 bits, the leading one among them
+  int hi = (int)(m >> 32) + ((1022 + 63 - lz) << 20) + s.hi_out;   // the leading one adds to the exponent
+  hi = a == 0 ? 0 : hi;
+  return __hiloint2double(hi | ((int)(sg) & 0x80000000) | s.poison, (int)m);
+}
+__device__ __forceinline__ cplx<double> from_work(cplx<long long> v, const Scale<double>& s) {
+  return {from_fx(v.x, s), from_fx(v.y, s)};
+}
+__device__ __forceinline__ cplx<float> from_work(cplx<float> v, const Scale<float>&) { return v; }
+// v / 2^s, rounded
+__device__ __forceinline__ long long fx_shift(long long v, long long half, int s) { return (v + half) >> s; }
+__device__ __forceinline__ cplx<long long> shifted(cplx<long long> v, int s) {
+  const long long half = (1ll << s) >> 1;
+  return {fx_shift(v.x, half, s), fx_shift(v.y, half, s)};
+}
+__device__ __forceinline__ cplx<long long> pass2(cplx<long long> v, const Scale<double>& s) { return shifted(v, s.s2); }
+__device__ __forceinline__ cplx<long long> pass3(cplx<long long> v, const Scale<double>& s) { return shifted(v, s.s3); }
+__device__ __forceinline__ cplx<float> pass2(cplx<float> v, const Scale<float>&) { return v; }
+__device__ __forceinline__ cplx<float> pass3(cplx<float> v, const Scale<float>&) { return v; }
+
+// v 2^-x from above, as a float (x: exponent of a bound on |v|, so that nothing overflows; the
+// conversion rounds up, so that nothing is lost at the other end).
+__device__ __forceinline__ float fx_float(double v, int x) {
+  const int hi = __double2hiint(v) & 0x7fffffff;
+  const int h = hi >= 0x7ff00000 ? hi : (hi > max(0, x << 20) || x < 0) && hi != 0 ? hi - (x << 20) : 0;
+  return __double2float_ru(__hiloint2double(h, __double2loint(v)));
+}
+// a 2^x
+__device__ __forceinline__ double fx_unscale(float a, int x) {
+  return x >= 1000 ? __hiloint2double(0x7ff00000, 0) : (double)a * __hiloint2double((x + 1023) << 20, 0);
+}
+
+// Bounds of a spectrum: the largest modulus and the sum of the moduli of the values added, in floats
+// scaled by 2^-x.
+struct SpecBound {
+  float m = 0.f, s = 0.f;
+  // |v| w, w >= 0 from above
+  __device__ __forceinline__ void add(cplx<double> v, float w, int x) {
+    const float a = __fmul_ru(__fadd_ru(fx_float(v.x, x), fx_float(v.y, x)), w);
+    m = (a <= m) ? m : a;   // a NaN is kept
+    s = __fadd_ru(s, a);
+  }
+};
+constexpr int kBoundBuf = 8 * 32;   // floats of shared memory for block_bounds of up to 4 bounds
+
+// Block-wide maxima and sums, returned to every thread.
+template <int NB> __device__ __forceinline__ void block_bounds(SpecBound (&b)[NB], float* buf) {
+  static_assert(2 * NB * 32 <= kBoundBuf, "bound buffer");
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    for (int o = 16; o > 0; o >>= 1) {
+      const float m = __shfl_xor_sync(0xffffffffu, b[i].m, o), s = __shfl_xor_sync(0xffffffffu, b[i].s, o);
+      b[i].m = (m <= b[i].m) ? b[i].m : m;
+      b[i].s = __fadd_ru(b[i].s, s);
+    }
+  }
+  __syncthreads();   // buf may still be read from the previous use
+  if (lane == 0) {
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      buf[(2 * i) * 32 + wid] = b[i].m;
+      buf[(2 * i + 1) * 32 + wid] = b[i].s;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    float m = 0.f, s = 0.f;
+    for (int w = 0; w < nw; ++w) {
+      const float x = buf[(2 * i) * 32 + w];
+      m = (x <= m) ? m : x;
+      s = __fadd_ru(s, buf[(2 * i + 1) * 32 + w]);
+    }
+    b[i].m = m;
+    b[i].s = s;
+  }
+}
+
+// Scale of the inverse transform of a spectrum given by value(c), c < n, as the work volume's scale
+// for LEN nonzero values per axis: the exponent of the largest component first, then the sum.
+template <typename T, int LEN, typename Value>
+__device__ __forceinline__ Scale<T> spectrum_scale(int n, Value value, float* buf) {
+  if constexpr (sizeof(T) == 8) {
+    int h = 0;
+    for (int c = threadIdx.x; c < n; c += blockDim.x) {
+      const cplx<double> v = value(c);
+      h = max(h, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
+    }
+    h = __reduce_max_sync(0xffffffffu, h);
+    int* ib = reinterpret_cast<int*>(buf);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    __syncthreads();
+    if (lane == 0) ib[wid] = h;
+    __syncthreads();
+    h = 0;
+    for (int w = 0; w < nw; ++w) h = max(h, ib[w]);
+    const int x = (h >> 20) - 1022 + 1;   // modulus below 2^x (two components)
+    SpecBound b[1];
+    for (int c = threadIdx.x; c < n; c += blockDim.x) b[0].add(value(c), 1.f, x);
+    block_bounds<1>(b, buf);
+    return fx_scale<T, LEN>(fx_unscale(b[0].m, x), fx_unscale(b[0].s, x));
+  } else {
+    return Scale<T>{};
+  }
+}
+
+// |u p| from above at compact index (c1, c2, c3), u a kernel-table value
+struct PBound {
+  float c[3], b[3][3], slop;
+};
+template <typename T> __device__ __forceinline__ PBound pbound_setup(const Params<T>& P, const T* dl) {
+  PBound q;
+  q.slop = 0.f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    q.c[d] = (float)dl[d];
+    float t = fabsf(q.c[d]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      q.b[a][d] = (float)P.Bm[a][d];
+      t += 24.f * fabsf(q.b[a][d]);
+    }
+    q.slop += t;
+  }
+  q.slop *= 1e-6f;   // float rounding of the components, against cancellation at small |p|
+  return q;
+}
+__device__ __forceinline__ float pbound(const PBound& q, double u, float m1, float m2, float m3) {
+  float p2 = 0.f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const float p = q.c[d] + m1 * q.b[0][d] + m2 * q.b[1][d] + m3 * q.b[2][d];
+    p2 = fmaf(p, p, p2);
+  }
+  return __fmul_ru(__double2float_ru(fabs(u)), sqrtf(p2) * 1.00001f + q.slop);
+}
+
+// Norms of the volumes a[v], v < count (blockIdx.x), into out: the 2-norm over the grid points and the
+// largest modulus (its components added, so both from above up to rounding).
+template <typename T, int N> __global__ void __launch_bounds__(256) k_norms(const cplx<T>* a, const cplx<T>* b, Norm* na, Norm* nb) {
+  const cplx<T>* v = (blockIdx.y == 0 ? a : b) + (size_t)blockIdx.x * N * N * N;
+  Norm* out = (blockIdx.y == 0 ? na : nb) + blockIdx.x;
+  double s = 0.0, m = 0.0;
+  for (int r = threadIdx.x; r < N * N * N; r += blockDim.x) {
+    const double t = fabs((double)v[r].x) + fabs((double)v[r].y);
+    s = fma(t, t, s);
+    m = (t <= m) ? m : t;
+  }
+  __shared__ double ss[8], sm[8];
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    const double t = __shfl_xor_sync(0xffffffffu, m, o);
+    m = (t <= m) ? m : t;
+  }
+  if ((threadIdx.x & 31) == 0) {
+    ss[threadIdx.x >> 5] = s;
+    sm[threadIdx.x >> 5] = m;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) {
+      s += ss[w];
+      m = (sm[w] <= m) ? m : sm[w];
+    }
+    out->two = sqrt(s);
+    out->inf = m;
+  }
+}
+
+}  // namespace tc

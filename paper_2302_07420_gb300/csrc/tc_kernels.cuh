@@ -10,6 +10,12 @@ constexpr int NT = 16;   // operator terms, order of TC_TERM_* in tc.h
 constexpr int kSmemLimit = 227 * 1024;   // bytes of shared memory per CTA on sm_103a
 enum { T2AH, T2BH1, T2BH2, T2AX, T2BX1, T2BX2, T3A1, T3A2, T3A3, T3A4, T3B1, T3B2, T3B3, T3B4, T3B5, T3B6 };
 
+// Norms of one real-space volume (fixed-point transforms, tc_fixed.cuh): its 2-norm over the grid
+// points and its largest modulus, from above.
+struct Norm {
+  double two, inf;
+};
+
 // Fields of one side.  Right side: ket = phi, bra = chi; left side: ket = chi,
 // bra = phi (Eq. BITCSCFconj).  Real-space fields are psi(r) = sum_G c(G) e^{iG.r}
 // on the unpadded n^3 grid.
@@ -22,6 +28,7 @@ template <typename T> struct SideArgs {
   cplx<T>* nt;           // [N]      FT[n] (1/N normalised)
   cplx<T>* mt;           // [3][N]   FT[m]
   cplx<T>* vH;           // [N]
+  cplx<T>* tn;           // [N]      tw3b6 n (over tw3b5 if P.fold), in the place of vH once k_vloc has read it
   cplx<T>* h1;           // [3][N]
   cplx<T>* vb2;          // [N]
   cplx<T>* t3b1;         // [N]
@@ -41,6 +48,8 @@ template <typename T> struct SideArgs {
   cplx<T>* v2;           // [nkb][4]  band points: V2_pp, V2_ap, V3_pp, V3_ap (see tc_band.cuh)
   cplx<T>* bh3a;         // [so][nkb no][3][N]  band points: h3 (3a4 kind) of their occupied orbitals
   cplx<T>* bh3b;         // [so][nkb no][3][N]  band points: h3 (3b kind)
+  // norms of ket and bra [Nkt nb], Y and w [nj_out][3], h3b [Nk no][3] and n (FP64 pruned kernels)
+  Norm *nket, *nbra, *nY, *nw, *nh3b, *nn;
   const T* tabV;         // [ndelta][2][N] -> this side's V at offset side*N
   T s2b;                 // +1 right, -1 left (sign of the grad u . grad terms)
   int side;
@@ -80,6 +89,7 @@ template <typename T> struct Params {
   int i2_0, nq2;         // occupied-pair stage: q2 items i2_0 .. i2_0 + nq2 - 1 (item = k no + mu)
   int h3_only;           // occupied-pair stage: the two h3 kinds only (parallel spins, no h6)
   int no_ap;             // pair stages without the work that reads only the antiparallel kernel table
+  int fold;              // the pruned pair chains run: Z carries f_q, Y and tn are over tw3b5 (if not 0)
   int band;              // outputs at band points: no SCF-mesh 3b6 corrections in k_finalize
   int nkb;               // band points (band contexts)
   const double* bandc;   // [nkb][4]: W (3), Gamma_b

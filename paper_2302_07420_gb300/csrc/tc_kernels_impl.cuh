@@ -78,6 +78,10 @@ __device__ __forceinline__ PComp<T> pcomp_setup(const Params<T>& P, const T* dl,
   q.b3 = d == 0 ? P.Bm[2][0] : (d == 1 ? P.Bm[2][1] : P.Bm[2][2]);
   return q;
 }
+// The constants of s p_d: a factor of every element at no cost per element.
+template <typename T> __device__ __forceinline__ PComp<T> scaled(const PComp<T>& q, T s) {
+  return PComp<T>{s * q.c0, s * q.b1, s * q.b2, s * q.b3};
+}
 
 template <typename T, int N> __device__ __forceinline__ T pcomp(const PComp<T>& q, int i1, int i2, int i3) {
   const T r1 = (T)(i1 <= (N - 1) / 2 ? i1 : i1 - N);
@@ -569,6 +573,7 @@ template <typename T, int N> __global__ void k_vloc(Params<T> P) {
     cplx<T> v = P.tw[T2AH] * S.vH[r] + (P.tw[T2BH2] * S.s2b) * S.vb2[r] - (T(0.5) * P.tw[T3A1]) * h1h1 +
                 (T(0.5) * P.tw[T3A2]) * S.h6[r] - P.tw[T3B1] * S.t3b1[r] + P.tw[T3B2] * S.t3b2[r];
     S.vloc[r] = v;
+    S.tn[r] = (P.fold ? P.tw[T3B6] / (P.tw[T3B5] != T(0) ? P.tw[T3B5] : T(1)) : P.tw[T3B6]) * S.n[r];   // in place of v_H
   }
 }
 
@@ -581,7 +586,10 @@ template <typename T, int N> __global__ void k_prep_zy(Params<T> P) {
   const size_t NN = (size_t)N * N * N;
   const size_t nz = (size_t)P.Nk * P.no * 3, ny = (size_t)P.nj_out * 3;
   const T* tw = P.tw;
-  const T zg = -S.s2b * tw[T2BX1], zh = -tw[T3A4], y1 = tw[T3B3], yg = -S.s2b * tw[T2BX2];
+  // for the pruned pair chains (P.fold) Z carries f_q and Y 1 / tw3b5, which saves them two
+  // products per grid point and component
+  const T iy = P.fold && tw[T3B5] != T(0) ? T(1) / tw[T3B5] : T(1);
+  const T zg = -S.s2b * tw[T2BX1], zh = -tw[T3A4], y1 = iy * tw[T3B3], yg = -S.s2b * iy * tw[T2BX2];
   const size_t total = (nz + ny) * NN;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const size_t v = e / NN, r = e % NN;
@@ -589,7 +597,8 @@ template <typename T, int N> __global__ void k_prep_zy(Params<T> P) {
       const size_t qd = v;                       // (k * no + mu) * 3 + d
       const size_t d = qd % 3, qo = qd / 3;
       const size_t q = (qo / P.no) * P.nb + qo % P.no;
-      S.Z[e] = zg * S.gket[(q * 3 + d) * NN + r] + zh * S.h3a4[e];
+      const cplx<T> z = zg * S.gket[(q * 3 + d) * NN + r] + zh * S.h3a4[e];
+      S.Z[e] = P.fold ? (T)(P.occ[q] / P.Nk) * z : z;
     } else {
       const size_t jd = v - nz, d = jd % 3, j = P.j0 + jd / 3;   // Y is indexed by j - j0
       S.Y[jd * NN + r] = y1 * (S.h1[d * NN + r] * S.ket[j * NN + r]) + yg * S.gket[(j * 3 + d) * NN + r];

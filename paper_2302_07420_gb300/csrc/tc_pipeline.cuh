@@ -20,7 +20,7 @@ template <typename T, int N> static void fill_side(tc_ctx* ctx, int side, SideAr
   cplx<T>* base = reinterpret_cast<cplx<T>*>(reinterpret_cast<char*>(ctx->d_side) + side * ctx->side_bytes);
   size_t o = 0;
   auto take = [&](size_t vols) { cplx<T>* p = base + o * NN; o += vols; return p; };
-  s.n = take(1); s.m = take(3); s.nt = take(1); s.mt = take(3); s.vH = take(1); s.h1 = take(3);
+  s.n = take(1); s.m = take(3); s.nt = take(1); s.mt = take(3); s.vH = take(1); s.tn = s.vH; s.h1 = take(3);
   s.vb2 = take(1); s.t3b1 = take(1); s.t3b2 = take(1); s.vu = take(2); s.spec = take(3); s.h5 = take(3);
   s.h6 = take(1); s.vloc = take(1);
   s.h3a4 = take((size_t)ctx->so_max * S.Nk * S.no * 3);
@@ -43,6 +43,18 @@ template <typename T, int N> static void fill_side(tc_ctx* ctx, int side, SideAr
   s.tabV = reinterpret_cast<const T*>(ctx->d_tabV);
   s.s2b = side == 0 ? T(1) : T(-1);
   s.side = side;
+  // norms: phi, chi, then per side n, Y, h3b, w.  Without their own buffer (tc_apply_noalloc) they sit in
+  // base fields that are dead by then: mt (phi and chi, written after the Hartree-type stage) and spec, h5,
+  // h6 (the rest, written after k_vloc)
+  const size_t no_all = (size_t)S.Nkt * S.nb, per = norms_per_side(ctx->nj_out, S.Nk, S.no);
+  Norm* np = ctx->d_norms ? ctx->d_norms : reinterpret_cast<Norm*>(ctx->d_side) + (size_t)5 * NN * sizeof(cplx<T>) / sizeof(Norm);
+  Norm* ns = ctx->d_norms ? ctx->d_norms + 2 * no_all + side * per : reinterpret_cast<Norm*>(s.spec);
+  s.nket = np + (side == 0 ? 0 : no_all);
+  s.nbra = np + (side == 0 ? no_all : 0);
+  s.nn = ns;
+  s.nY = ns + 1;
+  s.nh3b = s.nY + (size_t)ctx->nj_out * 3;
+  s.nw = s.nh3b + (size_t)S.Nk * S.no * 3;
 }
 
 template <typename T, int N> static Params<T> make_params(tc_ctx* ctx, const double* tw) {
@@ -156,6 +168,7 @@ template <typename T, int N> int prepare_kernels(tc_ctx* ctx) {
   // twiddles exp(-2 pi i j/L) for every codelet length, FP64 host sin/cos
   static double tw64[2 * kTwTotal];
   static float tw32[2 * kTwTotal];
+  static long long twfx[2 * kTwTotal];   // 2^63 w of the twiddles proper, in long double
   for (int i = 0, off = 0; i < kNumTwLens; ++i) {
     const int L = kTwLens[i];
     for (int j = 0; j < L; ++j) {
@@ -164,11 +177,16 @@ template <typename T, int N> int prepare_kernels(tc_ctx* ctx) {
       tw64[2 * (off + j) + 1] = std::sin(a);
       tw32[2 * (off + j)] = (float)std::cos(a);
       tw32[2 * (off + j) + 1] = (float)std::sin(a);
+      const long double al = -2.0L * 3.14159265358979323846264338327950288L * j / L, two63 = 9223372036854775808.0L;
+      const bool quarter = (4 * j) % L == 0;   // 1, -i, -1, i: never loaded
+      twfx[2 * (off + j)] = quarter ? 0 : (long long)std::nearbyint(std::cos(al) * two63);
+      twfx[2 * (off + j) + 1] = quarter ? 0 : (long long)std::nearbyint(std::sin(al) * two63);
     }
     off += L;
   }
   cudaError_t e1 = cudaMemcpyToSymbol(c_tw64, tw64, sizeof(tw64));
   cudaError_t e2 = cudaMemcpyToSymbol(c_tw32, tw32, sizeof(tw32));
+  if (e2 == cudaSuccess) e2 = cudaMemcpyToSymbol(c_twfx, twfx, sizeof(twfx));
   if (e1 != cudaSuccess || e2 != cudaSuccess) {
     ctx->err = "twiddle upload failed";
     return TC_ERR_CUDA;
@@ -292,6 +310,7 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   // pair densities whose spectra fit the compiled support take the pruned transforms
   constexpr int LP = kPruneL<N>;
   const bool pruned = LP < N && ctx->pair_support <= LP;
+  P.fold = pruned ? 1 : 0;
   // else, when they fit the distributed kernels' support, the cluster-distributed ones
   constexpr int LC = ClPlan<T, N>::L;
   using C0 = ClCfg<T, N, 0>;
@@ -302,6 +321,12 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   const bool dist_chain = dist && CLc > 0 && (ctx->cluster_ok & 1);
   const bool dist_3b4 = dist && CLb > 0 && (ctx->cluster_ok & 2);
   const bool dist_occ = dist && CLo > 0 && (ctx->cluster_ok & 4);
+  // FP64 pruned kernels run their transforms in fixed point, scaled by the norms of the fields
+  const bool fixed = sizeof(T) == 8 && pruned;
+  auto orbital_norms = [&] {
+    k_norms<T, N><<<dim3(nj_all, 2), 256, 0, st>>>((cplx<T>*)ctx->d_phi, (cplx<T>*)ctx->d_chi, P.side[0].nket,
+                                                   P.side[0].nbra);
+  };
   // 1. orbitals to real space
   stage_mark(ctx, st, 0);
   k_orbitals<T, N><<<dim3(nj_all, 4, 2), TH, vb1, st>>>(cphi, cchi, bphi, bchi, nj, ctx->d_box_index, ctx->d_kpg,
@@ -341,6 +366,10 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
     nl[1] = 0;
     nl[2] = 1;
     stage_mark(ctx, st, 2);
+    if (fixed) {
+      orbital_norms();
+      nl[2] += 1;
+    }
     k_prep_zy<T, N><<<dim3(2 * pw_blocks, nsides), 256, 0, st>>>(P);
     TC_CHECK_LAUNCH("k_prep_zy");
   } else {
@@ -370,6 +399,10 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   }
   // 3. occupied-pair stage
   stage_mark(ctx, st, 2);
+  if (fixed) {
+    orbital_norms();
+    nl[2] += 1;
+  }
   const bool need_a4 = tw[T3A2] != 0 || tw[T3A4] != 0 || tw[T3B2] != 0 || tw[T3B5] != 0;
   if (need_a4) {
     // two-sided launches compute the right side only and conjugate it into the left one when
@@ -457,6 +490,17 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   TC_CHECK_LAUNCH("k_prep_zy");
   nl[2] += 2;
   }
+  if (fixed) {
+    // tw3b6 n and, contiguous per side where they were written, Y and h3b (part 0)
+    for (int sd = 0; sd < nsides; ++sd) {
+      const SideArgs<T>& D = P.side[sd];
+      k_norms<T, N><<<dim3(1, 1), 256, 0, st>>>(D.tn, D.tn, D.nn, D.nn);
+      k_norms<T, N><<<dim3(P.nj_out * 3, 1), 256, 0, st>>>(D.Y, D.Y, D.nY, D.nY);
+      k_norms<T, N><<<dim3(S.Nk * S.no * 3, 1), 256, 0, st>>>(D.h3b, D.h3b, D.nh3b, D.nh3b);
+    }
+    TC_CHECK_LAUNCH("k_norms");
+    nl[2] += 3 * nsides;
+  }
   // 4. pair chains (with symmetry: output orbitals of irreducible k-points only)
   stage_mark(ctx, st, 3);
   const int nj_items = P.sym ? P.nirr * S.nb : P.nj_out;
@@ -499,6 +543,12 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
       k_band_scalars<T, N><<<dim3(S.nkb * S.no * S.nb, 2), 256, 0, st>>>(P, 2);
       TC_CHECK_LAUNCH("band w_c");
       nl[4] += 2;
+    }
+    if (fixed && tw[T3B4] != 0) {
+      for (int sd = 0; sd < nsides; ++sd)
+        k_norms<T, N><<<dim3(P.nj_out * 3, 1), 256, 0, st>>>(P.side[sd].w, P.side[sd].w, P.side[sd].nw, P.side[sd].nw);
+      TC_CHECK_LAUNCH("k_norms");
+      nl[4] += nsides;
     }
     Params<T> Pb = P;
     Pb.nsmem = smem_vols<T, N>(2);
