@@ -365,8 +365,9 @@ size_t side_field_vols(int Nk, int nb, int no, int so_max, int sc_max, int nj_ou
 
 // Number of partner chunks s for a launch of `items` CTA items (per chunk one CTA): the s
 // (1 <= s <= min(8, partners)) that fills the last wave of CTAs over the SMs best, the
-// smallest such s when several are within 1 %.
-void choose_splits(tc_ctx* c) {
+// smallest such s when several are within 1 %.  small: more chunks where so few items leave SMs idle
+// (pick_split_small).
+void choose_splits(tc_ctx* c, bool small) {
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || sms <= 0) {
     cudaGetLastError();
@@ -375,8 +376,8 @@ void choose_splits(tc_ctx* c) {
   const Setup& S = c->S;
   const int M = S.Nk * S.no, nj = c->nj_out;
   for (int sides = 1; sides <= 2; ++sides) {
-    c->split_occ[sides - 1] = pick_split(M * sides, M, sms);
-    c->split_chain[sides - 1] = pick_split(nj * sides, M, sms);
+    c->split_occ[sides - 1] = small ? pick_split_small(M * sides, M, sms) : pick_split(M * sides, M, sms);
+    c->split_chain[sides - 1] = small ? pick_split_small(nj * sides, M, sms) : pick_split(nj * sides, M, sms);
   }
   c->so_max = std::max(c->split_occ[0], c->split_occ[1]);
   c->sc_max = std::max(c->split_chain[0], c->split_chain[1]);

@@ -78,10 +78,10 @@ template <typename T, int N> struct ClPlan {
     if (sizeof(T) == 8) return choice64(kind);
     switch (N) {
       case 24: return kind == 0 ? ClChoice{2, 1, 1, 0, 4} : ClChoice{2, 1, 1, 0, 1};
-      case 25: return kind == 0 ? ClChoice{2, 1, 1, 0, 4} : (kind == 1 ? ClChoice{2, 1, 1, 0, 1} : ClChoice{2, 0, 1, 0, 1, 1});
+      case 25: return kind == 0 ? ClChoice{2, 1, 1, 0, 1} : (kind == 1 ? ClChoice{2, 1, 1, 0, 1} : ClChoice{2, 0, 1, 0, 1, 1});
       case 27: return kind == 0 ? ClChoice{2, 1, 1, 0, 2} : (kind == 1 ? ClChoice{2, 1, 1, 0, 1} : ClChoice{2, 0, 1, 0, 1});
-      case 30: return kind == 0 ? ClChoice{2, 2, 1, 0, 1} : (kind == 1 ? ClChoice{2, 1, 1, 0, 1} : ClChoice{2, 0, 1, 0, 1});
-      case 32: return kind == 0 ? ClChoice{2, 2, 1, 0, 1} : (kind == 1 ? ClChoice{2, 1, 1, 0, 1} : ClChoice{3, 0, 1, 0, 1});
+      case 30: return kind == 0 ? ClChoice{2, 2, 1, 0, 2} : (kind == 1 ? ClChoice{2, 1, 1, 0, 1} : ClChoice{2, 0, 1, 0, 1});
+      case 32: return kind == 0 ? ClChoice{2, 2, 1, 0, 2} : (kind == 1 ? ClChoice{2, 1, 1, 0, 1} : ClChoice{3, 0, 1, 0, 1});
       case 48: return kind == 0 ? ClChoice{4, 0, 1, 288, 4} : (kind == 1 ? ClChoice{6, 0, 1, 0, 1} : ClChoice{8, 0, 1, 0, 1});
       default: return ClChoice{0, 0, 0, 0, 1};
     }
@@ -283,6 +283,9 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
   const bool need_F = need_y || tw[T3B5] != T(0) || tw[T3B6] != T(0);
   const bool need_ap = tw[T3B6] != T(0) && !P.no_ap;
   const T t3b5 = tw[T3B5], t3b6 = tw[T3B6], t2ax = tw[T2AX];
+  // weights folded as in k_pair_chain_pr: Z carries f, Y and n are over tw3b5
+  const bool all = need_z && need_w && need_y && t3b5 != T(0) && t3b6 != T(0);
+  const T g35 = t3b5 != T(0) ? t3b5 : T(1);
   for (int r = rank * blockDim.x + threadIdx.x; r < (int)NN; r += CL * blockDim.x) {
     acc[r] = cplx<T>{0, 0};
     for (int d = 0; d < 3; ++d) w[d * NN + r] = cplx<T>{0, 0};
@@ -291,8 +294,9 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
   for (int qi = qi_begin; qi < qi_end; ++qi) {
     const int kq = qi / P.no, mu = qi % P.no;
     const int q = kq * P.nb + mu;
-    const T f = (T)(P.occ[q] / P.Nk);
+    const T f = weight(P, q);
     if (f == T(0)) continue;
+    const T ft2ax = f * t2ax;
     const int did = P.delta_id[kj * P.kstride + kq];
     const T* dl = P.delta + did * 3;
     const T* Vt = SD.tabV + ((size_t)did * 2 + SD.side) * NN;
@@ -365,7 +369,7 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
       if (sp == 1 && !need_ap) continue;
       for (int d = 0; d < 3; ++d) {
         const bool first_C = (sp == 0 && d == 0);
-        const PComp<T> qd = pcomp_setup<T>(P, dl, d);
+        const PComp<T> qd = pcomp_setup<T>(P, dl, d), qf = scaled(qd, g35 * P.invN);
         // b = FT^{-1}[U_d A]
         cinv_23<T, N, L, CL>(cluster, B, c1_0, nrow, [&](int r, int c1, int c2, int c3) {
           return mul_si<T, 1>((pcomp_c<T, N, L>(qd, c1, c2, c3) * tab(sp, r, c1, c2, c3)) * A[D::cidx(r, c2, c3)]);
@@ -375,42 +379,50 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
             cluster, rb, rank, [&](int, int, int) { return cplx<T>{0, 0}; },
             [&](int, int i2, int i3, cplx<T>(&v)[N]) {
               if (sp == 0) {
+                if (all) {
+                  // CH points at a time, their loads issued before any of their reductions
 #pragma unroll
-                for (int c0 = 0; c0 < N; c0 += CH) {
-                  cplx<T> lz[CH], lk[CH], ly[CH], lb[CH], lj[CH], lh[CH], ln[CH];
+                  for (int c0 = 0; c0 < N; c0 += CH) {
+                    cplx<T> lz[CH], lk[CH], ly[CH], lb[CH], lj[CH], lh[CH], ln[CH];
 #pragma unroll
-                  for (int u = 0; u < CH; ++u) {
-                    if (c0 + u >= N) continue;
-                    const int g = G::gidx(c0 + u, i2, i3);
-                    if (need_z) lz[u] = ldg(Zq + d * NN + g);
-                    lk[u] = ldg(ketq + g);
-                    if (need_F) {
+                    for (int u = 0; u < CH; ++u) {
+                      if (c0 + u >= N) continue;
+                      const int g = G::gidx(c0 + u, i2, i3);
+                      lz[u] = ldg(Zq + d * NN + g);
+                      lk[u] = ldg(ketq + g);
                       ly[u] = ldg(Yj + d * NN + g);
                       lb[u] = ldg(braq + g);
                       lj[u] = ldg(ketj + g);
                       lh[u] = ldg(h3bq + d * NN + g);
-                      ln[u] = ldg(SD.n + g);
+                      ln[u] = ldg(SD.tn + g);
+                    }
+#pragma unroll
+                    for (int u = 0; u < CH; ++u) {
+                      if (c0 + u >= N) continue;
+                      const int g = G::gidx(c0 + u, i2, i3);
+                      const cplx<T> bv = v[c0 + u];
+                      red_add_v(&acc[g], lz[u] * bv);
+                      red_add_v(&w[d * NN + g], f * (lk[u] * bv));
+                      v[c0 + u] = ln[u] * bv + mulc(ly[u], lb[u]) - lj[u] * lh[u];   // F / g35
                     }
                   }
+                } else {   // some of the terms are off
 #pragma unroll
-                  for (int u = 0; u < CH; ++u) {
-                    if (c0 + u >= N) continue;
-                    const int g = G::gidx(c0 + u, i2, i3);
-                    const cplx<T> bv = v[c0 + u];
-                    if (need_z) red_add_v(&acc[g], f * (lz[u] * bv));
-                    if (need_w) red_add_v(&w[d * NN + g], f * (lk[u] * bv));
+                  for (int i = 0; i < N; ++i) {
+                    const int g = G::gidx(i, i2, i3);
+                    const cplx<T> bv = v[i];
+                    if (need_z) red_add_v(&acc[g], ldg(Zq + d * NN + g) * bv);
+                    if (need_w) red_add_v(&w[d * NN + g], f * (ldg(ketq + g) * bv));
                     cplx<T> F = {0, 0};
-                    if (need_F) {
-                      if (need_y) F = mulc(ly[u], lb[u]);
-                      if (t3b5 != T(0)) F = F - t3b5 * (lj[u] * lh[u]);
-                      if (t3b6 != T(0)) F = F + t3b6 * (ln[u] * bv);
-                    }
-                    v[c0 + u] = F;
+                    if (t3b6 != T(0)) F = ldg(SD.tn + g) * bv;
+                    if (need_y) F = F + mulc(ldg(Yj + d * NN + g), ldg(braq + g));
+                    if (t3b5 != T(0)) F = F - ldg(ketj + g) * ldg(h3bq + d * NN + g);
+                    v[i] = F;
                   }
                 }
               } else {
 #pragma unroll
-                for (int i = 0; i < N; ++i) v[i] = t3b6 * (ldg(SD.n + G::gidx(i, i2, i3)) * v[i]);
+                for (int i = 0; i < N; ++i) v[i] = ldg(SD.tn + G::gidx(i, i2, i3)) * v[i];
               }
             },
             fwd);
@@ -418,10 +430,10 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
         // C += -U_d FT[F] = -i p_d u FT[F]; a cinv_23 always follows (the next component's or the
         // final one: C is then nonzero), so a CTA barrier closes the pass
         cfwd_32<T, N, L, CL, false>(cluster, B, c1_0, nrow, [&](int r, int c1, int c2, int c3, cplx<T> v) {
-          const T k = pcomp_c<T, N, L>(qd, c1, c2, c3) * tab(sp, r, c1, c2, c3) * P.invN;
-          const cplx<T> t = mul_si<T, -1>(k * v);
+          const T k = pcomp_c<T, N, L>(qf, c1, c2, c3) * tab(sp, r, c1, c2, c3);
           const int s = D::cidx(r, c2, c3);
-          C[s] = first_C ? t : C[s] + t;
+          const cplx<T> c0 = first_C ? cplx<T>{0, 0} : C[s];
+          C[s] = cplx<T>{fma(k, v.y, c0.x), fma(-k, v.x, c0.y)};   // C -= i k v
         });
       }
     }
@@ -429,8 +441,8 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
     if (has_C || t2ax != T(0)) {
       cinv_23<T, N, L, CL>(cluster, B, c1_0, nrow, [&](int r, int c1, int c2, int c3) {
         const int s = D::cidx(r, c2, c3);
-        cplx<T> v = has_C ? C[s] : cplx<T>{0, 0};
-        if (t2ax != T(0)) v = v - (t2ax * tab(2, r, c1, c2, c3)) * A[s];
+        cplx<T> v = has_C ? f * C[s] : cplx<T>{0, 0};
+        if (t2ax != T(0)) v = v - (ft2ax * tab(2, r, c1, c2, c3)) * A[s];
         return v;
       });
       caxis1<T, N, L, CL, true>(
@@ -444,7 +456,7 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
                 if (c0 + u < N) lk[u] = ldg(ketq + G::gidx(c0 + u, i2, i3));
 #pragma unroll
               for (int u = 0; u < 4; ++u)
-                if (c0 + u < N) red_add_v(&acc[G::gidx(c0 + u, i2, i3)], f * (lk[u] * v[c0 + u]));
+                if (c0 + u < N) red_add_v(&acc[G::gidx(c0 + u, i2, i3)], lk[u] * v[c0 + u]);
             }
           },
           false);
@@ -498,7 +510,7 @@ __global__ void __launch_bounds__(ClCfg<T, N, 1>::threads, ClCfg<T, N, 1>::MINB)
   for (int qi = qi_begin; qi < qi_end; ++qi) {
     const int kq = qi / P.no, mu = qi % P.no;
     const int q = kq * P.nb + mu;
-    const T f = (T)(P.occ[q] / P.Nk);
+    const T f = weight(P, q);
     if (f == T(0)) continue;
     const int did = P.delta_id[kj * P.kstride + kq];
     const T* dl = P.delta + did * 3;
@@ -601,7 +613,7 @@ __global__ void __launch_bounds__(ClCfg<T, N, 2>::threads, ClCfg<T, N, 2>::MINB)
 #pragma unroll
   for (int k = 0; k < CL; ++k) rb[k] = cluster.map_shared_rank(W, k);
   const size_t NN = G::nn;
-  const T f2 = (T)(P.occ[q2] / P.Nk);
+  const T f2 = weight(P, q2);
   cplx<T>* h3a4 = SD.h3a4 + ((size_t)chunk * P.nq2 + (i2 - P.i2_0)) * 3 * NN;
   cplx<T>* h3b = SD.h3b + ((size_t)chunk * P.nq2 + (i2 - P.i2_0)) * 3 * NN;
   const cplx<T>* bra2 = SD.bra + (size_t)q2 * NN;
@@ -623,7 +635,7 @@ __global__ void __launch_bounds__(ClCfg<T, N, 2>::threads, ClCfg<T, N, 2>::MINB)
   for (int i1 = i1_begin; i1 < i1_end; ++i1) {
     const int k1 = i1 / P.no, mu1 = i1 % P.no;
     const int q1 = k1 * P.nb + mu1;
-    const T f1 = (T)(P.occ[q1] / P.Nk);
+    const T f1 = weight(P, q1);
     if (f1 == T(0) || f2 == T(0)) continue;
     const int id12 = P.delta_id[k2 * P.kstride + k1];   // Delta = k2 - k1 -> for P(q1,q2)
     const int id21 = P.delta_id[k1 * P.kstride + k2];   // Delta = k1 - k2 -> for P(q2,q1)

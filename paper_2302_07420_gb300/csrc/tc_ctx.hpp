@@ -136,7 +136,7 @@ constexpr int kBandScalars = 13;
 void destroy_context(tc_ctx* c);
 WsLayout ws_layout(const tc_ctx* c);
 // Chooses the partner-chunk counts of c for the current device (needs c->S).
-void choose_splits(tc_ctx* c);
+void choose_splits(tc_ctx* c, bool small = true);
 // n^3 volumes of one side's field block (see fill_side).
 size_t side_field_vols(int Nk, int nb, int no, int so_max, int sc_max, int nj_out, int nkb, int so_band);
 // Norms of one side: n, Y, h3b, w (see fill_side).

@@ -222,6 +222,38 @@ __device__ __forceinline__ float pbound(const PBound& q, double u, float m1, flo
   return __fmul_ru(__double2float_ru(fabs(u)), sqrtf(p2) * 1.00001f + q.slop);
 }
 
+// 3D transforms of one volume per CTA (fwd3d, inv3d of tc_fft.cuh; same arguments) in fixed point where
+// the FP64 volume is in shared memory: their latency is that of one CTA on one SM's FP64 pipe
+// otherwise.  The values go into the volume first and the scale is taken from there: a load may be 25 FP64
+// operations, which are done once.  buf: kBoundBuf floats.
+template <typename T, int N> constexpr bool kFxVolume = sizeof(T) == 8 && (size_t)Geo<N>::vol * sizeof(cplx<T>) + 1024 <= (size_t)kSmemLimit;
+
+template <typename T, int N, bool FWD, typename Load, typename Emit>
+__device__ __forceinline__ void volume3d(cplx<T>* V, Load load, Emit emit, float* buf) {
+  using G = Geo<N>;
+  if constexpr (kFxVolume<T, N>) {
+    using I = long long;
+    constexpr int S = FWD ? -1 : +1, A1 = FWD ? 1 : 2, A3 = FWD ? 2 : 1;
+    auto at = [](int c) { return G::sidx(c / (N * N), (c / N) % N, c % N); };
+#pragma unroll 2
+    for (int c = threadIdx.x; c < G::nn; c += blockDim.x) V[at(c)] = load(c / (N * N), (c / N) % N, c % N);
+    // (each thread takes the maximum and the sum over the points that it stored itself)
+    const Scale<T> sc = spectrum_scale<T, N>(G::nn, [&](int c) { return V[at(c)]; }, buf);
+    cplx<I>* W = reinterpret_cast<cplx<I>*>(V);
+    auto put = [&](int a, int b, int c, cplx<I> v) { W[G::sidx(a, b, c)] = v; };
+    fft_pass<I, N, S, A1>([&](int a, int b, int c) { return to_work(V[G::sidx(a, b, c)], sc); }, put);
+    __syncthreads();
+    fft_pass<I, N, S, 3>([&](int a, int b, int c) { return pass2(W[G::sidx(a, b, c)], sc); }, put);
+    __syncthreads();
+    fft_pass<I, N, S, A3>([&](int a, int b, int c) { return pass3(W[G::sidx(a, b, c)], sc); },
+                          [&](int a, int b, int c, cplx<I> v) { emit(a, b, c, from_work(v, sc)); });
+  } else if constexpr (FWD) {
+    fwd3d<T, N>(V, load, emit);
+  } else {
+    inv3d<T, N>(V, load, emit);
+  }
+}
+
 // Norms of the volumes a[v], v < count (blockIdx.x), into out: the 2-norm over the grid points and the
 // largest modulus (its components added, so both from above up to rounding).
 template <typename T, int N> __global__ void __launch_bounds__(256) k_norms(const cplx<T>* a, const cplx<T>* b, Norm* na, Norm* nb) {

@@ -17,7 +17,7 @@
 //   k_local        local terms and 3b6 corrections (Eqs. 3b6_div_scf1/2/3; scalars: k_corr_scalars)
 //   k_finalize     FFT, box -> sphere
 #pragma once
-#include "tc_kernels.cuh"
+#include "tc_fixed.cuh"
 
 namespace tc {
 
@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
                const double* __restrict__ kpg, int npw_max, int nb, cplx<T>* phi, cplx<T>* chi, cplx<T>* gphi,
                cplx<T>* gchi, cplx<T>* gwork) {
   using G = Geo<N>;
+  __shared__ float bbuf[kFxVolume<T, N> ? kBoundBuf : 1];
   extern __shared__ __align__(16) unsigned char smraw[];
   cplx<T>* V = work_vol<T, N>(smraw, gwork);
   const int j = blockIdx.x, comp = blockIdx.y, set = blockIdx.z;
@@ -159,8 +160,8 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
   __syncthreads();
   cplx<T>* dst = comp == 0 ? (set == 0 ? phi : chi) + (size_t)j * G::nn
                            : (set == 0 ? gphi : gchi) + ((size_t)j * 3 + (comp - 1)) * G::nn;
-  inv3d<T, N>(V, [&](int a, int b, int cc) { return V[G::sidx(a, b, cc)]; },
-              [&](int a, int b, int cc, cplx<T> v) { dst[G::gidx(a, b, cc)] = v; });
+  volume3d<T, N, false>(V, [&](int a, int b, int cc) { return V[G::sidx(a, b, cc)]; },
+                        [&](int a, int b, int cc, cplx<T> v) { dst[G::gidx(a, b, cc)] = v; }, bbuf);
 }
 
 // BF16 storage (TC_BF16_STORE): every value of a[0 .. n) rounded to the nearest BF16 (ties to even),
@@ -184,7 +185,7 @@ template <typename T, int N> __global__ void k_density(Params<T> P) {
     for (int k = 0; k < P.Nk; ++k)
       for (int mu = 0; mu < P.no; ++mu) {
         const int q = k * P.nb + mu;
-        const T f = (T)(P.occ[q] / P.Nk);
+        const T f = weight(P, q);
         if (f == T(0)) continue;
         const cplx<T> b = conjg(S.bra[(size_t)q * NN + r]);
         n = n + f * (b * S.ket[(size_t)q * NN + r]);
@@ -206,6 +207,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(Cfg<N>::threads)
     k_spec_fwd(Params<T> P, int which) {
   using G = Geo<N>;
+  __shared__ float bbuf[kFxVolume<T, N> ? kBoundBuf : 1];
   extern __shared__ __align__(16) unsigned char smraw[];
   cplx<T>* V = work_vol<T, N>(smraw, P.scratch);
   const SideArgs<T>& S = P.side[blockIdx.y];
@@ -220,13 +222,13 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
   } else {                   // FT[h5_c]    (Alg. 8)
     a = S.h5 + (size_t)c * G::nn; dst = S.spec + (size_t)c * G::nn;
   }
-  fwd3d<T, N>(
+  volume3d<T, N, true>(
       V,
       [&](int i, int j, int k) {
         cplx<T> v = a[G::gidx(i, j, k)];
         return b ? v * b[G::gidx(i, j, k)] : v;
       },
-      [&](int i, int j, int k, cplx<T> v) { dst[G::gidx(i, j, k)] = P.invN * v; });
+      [&](int i, int j, int k, cplx<T> v) { dst[G::gidx(i, j, k)] = P.invN * v; }, bbuf);
 }
 
 // Hartree-type convolutions (Delta = 0, G = 0 dropped), blockIdx.y = side.
@@ -243,6 +245,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(Cfg<N>::threads)
     k_hartree_inv(Params<T> P, int kind_or_all) {
   using G = Geo<N>;
+  __shared__ float bbuf[kFxVolume<T, N> ? kBoundBuf : 1];
   extern __shared__ __align__(16) unsigned char smraw[];
   cplx<T>* V = work_vol<T, N>(smraw, P.scratch);
   const SideArgs<T>& S = P.side[blockIdx.y];
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
   const PComp<T> qc = pcomp_setup<T>(P, nullptr, kind == 1 ? c : 0);
   cplx<T>* dst = kind == 0 ? S.vH : kind == 1 ? S.h1 + (size_t)c * G::nn : kind == 2 ? S.vb2 : kind == 3 ? S.t3b1
                : kind == 4 ? S.t3b2 : S.vu + (size_t)c * G::nn;
-  inv3d<T, N>(
+  volume3d<T, N, false>(
       V,
       [&](int i, int j, int k) {
         const int g = G::gidx(i, j, k);
@@ -273,7 +276,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
         for (int d = 0; d < 3; ++d) s = s + (p[d] * u) * src[(size_t)d * G::nn + g];
         return mul_si<T, -1>(s);   // -i G u . src
       },
-      [&](int i, int j, int k, cplx<T> v) { dst[G::gidx(i, j, k)] = v; });
+      [&](int i, int j, int k, cplx<T> v) { dst[G::gidx(i, j, k)] = v; }, bbuf);
 }
 
 // ---------------------------------------------------------------------------
@@ -307,7 +310,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads, 1) k_occ_pairs(Params<T> P) {
   cplx<T>* H6 = vol_slot<T, N>(P, sm, 4, NS, true);
   cplx<T>* FAB = vol_slot<T, N>(P, sm, 5, NS, true);
   const size_t NN = G::nn;
-  const T f2 = (T)(P.occ[q2] / P.Nk);
+  const T f2 = weight(P, q2);
   cplx<T>* h3a4 = S.h3a4 + ((size_t)chunk * P.nq2 + (i2 - P.i2_0)) * 3 * NN;
   cplx<T>* h3b = S.h3b + ((size_t)chunk * P.nq2 + (i2 - P.i2_0)) * 3 * NN;
   const cplx<T>* bra2 = S.bra + (size_t)q2 * NN;
@@ -330,7 +333,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads, 1) k_occ_pairs(Params<T> P) {
     const T* d21 = P.delta + id21 * 3;
     {
       const int q1 = k1 * P.nb + mu1;
-      const T f1 = (T)(P.occ[q1] / P.Nk);
+      const T f1 = weight(P, q1);
       if (f1 == T(0) || f2 == T(0)) continue;
       const cplx<T>* bra1 = S.bra + (size_t)q1 * NN;
       const cplx<T>* ket1 = S.ket + (size_t)q1 * NN;
@@ -471,7 +474,7 @@ template <typename T, int N> __global__ void k_reduce_a4(Params<T> P, int side0,
     for (int c = 0; c < M; ++c) {
       const int k = c / P.no, mu = c % P.no;
       const int q = k * P.nb + mu;
-      const T f = (T)(P.occ[q] / P.Nk);
+      const T f = weight(P, q);
       const cplx<T> kv = S.ket[(size_t)q * NN + r];
 #pragma unroll
       for (int d = 0; d < 3; ++d) h5[d] = h5[d] + f * (S.h3b[((size_t)c * 3 + d) * NN + r] * kv);
@@ -598,7 +601,7 @@ template <typename T, int N> __global__ void k_prep_zy(Params<T> P) {
       const size_t d = qd % 3, qo = qd / 3;
       const size_t q = (qo / P.no) * P.nb + qo % P.no;
       const cplx<T> z = zg * S.gket[(q * 3 + d) * NN + r] + zh * S.h3a4[e];
-      S.Z[e] = P.fold ? (T)(P.occ[q] / P.Nk) * z : z;
+      S.Z[e] = P.fold ? weight(P, q) * z : z;
     } else {
       const size_t jd = v - nz, d = jd % 3, j = P.j0 + jd / 3;   // Y is indexed by j - j0
       S.Y[jd * NN + r] = y1 * (S.h1[d * NN + r] * S.ket[j * NN + r]) + yg * S.gket[(j * 3 + d) * NN + r];
@@ -665,7 +668,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads, 1) k_pair_chain(Params<T> P) 
     const T* Uap = P.tabU + ((size_t)did * 2 + 1) * NN;
     {
       const int q = kq * P.nb + mu;
-      const T f = (T)(P.occ[q] / P.Nk);
+      const T f = weight(P, q);
       if (f == T(0)) continue;
       const cplx<T>* braq = S.bra + (size_t)q * NN;
       const cplx<T>* ketq = S.ket + (size_t)q * NN;
@@ -831,7 +834,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads, 1) k_pair_3b4(Params<T> P) {
     const T* Upp = P.tabU + ((size_t)did * 2 + 0) * NN;
     {
       const int q = kq * P.nb + mu;
-      const T f = (T)(P.occ[q] / P.Nk);
+      const T f = weight(P, q);
       if (f == T(0)) continue;
       const cplx<T>* braq = S.bra + (size_t)q * NN;
       const cplx<T>* ketq = S.ket + (size_t)q * NN;
@@ -874,9 +877,9 @@ template <typename T, int N> __global__ void k_corr_scalars(Params<T> P) {
     const int item = e / P.no, mu = e % P.no;
     const int jo = P.sym ? P.irr[item / P.nb] * P.nb + item % P.nb : item;
     double* cs = S.cs + ((size_t)jo * P.no + mu) * 6;
-    const double f = P.occ[(P.j0 + jo) / P.nb * P.nb + mu], fq = f * P.invOm2;
+    const double fq = P.occ[(P.j0 + jo) / P.nb * P.nb + mu] * P.invOm2;
     cplx<T>* o = reinterpret_cast<cplx<T>*>(cs);
-    if ((T)(f / P.Nk) == T(0)) {   // the chains skip such a partner: its sums are unwritten
+    if (weight(P, (P.j0 + jo) / P.nb * P.nb + mu) == T(0)) {   // the chains skip such a partner: its sums are unwritten
       o[0] = o[1] = cplx<T>{0, 0};
       continue;
     }
@@ -937,6 +940,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(Cfg<N>::threads)
     k_finalize(Params<T> P, double2* outR, double2* outL, const int* __restrict__ box_index) {
   using G = Geo<N>;
+  __shared__ float bbuf[kFxVolume<T, N> ? kBoundBuf : 1];
   extern __shared__ __align__(16) unsigned char smraw[];
   cplx<T>* V = work_vol<T, N>(smraw, P.scratch);
   const int side = blockIdx.y;
@@ -946,8 +950,8 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
   const int jo = P.sym ? P.irr[blockIdx.x / P.nb] * P.nb + blockIdx.x % P.nb : blockIdx.x;
   const int kj = (P.j0 + jo) / P.nb;
   const cplx<T>* acc = S.acc + (size_t)jo * G::nn;
-  fwd3d<T, N>(V, [&](int a, int b, int c) { return ldg(acc + G::gidx(a, b, c)); },
-              [&](int a, int b, int c, cplx<T> v) { V[G::sidx(a, b, c)] = P.invN * v; });
+  volume3d<T, N, true>(V, [&](int a, int b, int c) { return ldg(acc + G::gidx(a, b, c)); },
+                       [&](int a, int b, int c, cplx<T> v) { V[G::sidx(a, b, c)] = P.invN * v; }, bbuf);
   __syncthreads();
   double2* o = out + (size_t)jo * P.npw_max;
   for (int g = threadIdx.x; g < P.npw_max; g += blockDim.x) {

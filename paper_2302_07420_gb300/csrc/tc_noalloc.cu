@@ -177,6 +177,10 @@ extern "C" tc_status tc_apply_noalloc(const tc_params* params, const void* phi_R
   }
   tc::choose_splits(&c);
   Layout L = plan(c, rsz);
+  if (L.total > kNoallocBytes) {
+    tc::choose_splits(&c, false);
+    L = plan(c, rsz);
+  }
   if (L.total > kNoallocBytes) {   // partner chunks multiply the accumulators: fall back to one chunk
     c.split_occ[0] = c.split_occ[1] = c.split_chain[0] = c.split_chain[1] = 1;
     c.so_max = c.sc_max = 1;

@@ -67,6 +67,7 @@ template <typename T, int N> static Params<T> make_params(tc_ctx* ctx, const dou
   P.invN = (T)(1.0 / ((double)N * N * N));
   P.Omega = S.Omega;
   P.invOm2 = 1.0 / (S.Omega * S.Omega);
+  P.invNk = 1.0 / S.Nk;
   for (int s = 0; s < 2; ++s) { P.corr_c[s] = S.corr_c[s]; P.A[s] = S.amp[s]; }
   for (int t = 0; t < NT; ++t) P.tw[t] = (T)tw[t];
   P.delta_id = ctx->d_delta_id;
@@ -198,9 +199,15 @@ template <typename T, int N> int prepare_kernels(tc_ctx* ctx) {
   TC_SET_SMEM((k_hartree_inv<T, N>), vb1);
   TC_SET_SMEM((k_finalize<T, N>), vb1);
   TC_SET_SMEM((k_band_v2<T, N>), vb1);
-  TC_SET_SMEM((k_occ_pairs<T, N>), (smem_vols<T, N>(4) * vb));
-  TC_SET_SMEM((k_pair_chain<T, N>), (smem_vols<T, N>(3) * vb));
-  TC_SET_SMEM((k_pair_3b4<T, N>), (smem_vols<T, N>(2) * vb));
+  if constexpr (!kFullPr<N>) {
+    TC_SET_SMEM((k_occ_pairs<T, N>), (smem_vols<T, N>(4) * vb));
+    TC_SET_SMEM((k_pair_chain<T, N>), (smem_vols<T, N>(3) * vb));
+    TC_SET_SMEM((k_pair_3b4<T, N>), (smem_vols<T, N>(2) * vb));
+  } else {
+    TC_SET_SMEM((k_pair_chain_pr<T, N, N>), (int)(PrSmem<T, N, N, 2, 3>::bytes));
+    TC_SET_SMEM((k_pair_3b4_pr<T, N, N>), (int)(PrSmem<T, N, N, 1, 1>::bytes));
+    TC_SET_SMEM((k_occ_pairs_pr<T, N, N>), (int)(OccSmem<T, N, N>::bytes));
+  }
   if constexpr (kPruneL<N> < N) {
     TC_SET_SMEM((k_pair_chain_pr<T, N, kPruneL<N>>), (int)(PrSmem<T, N, kPruneL<N>, 2, 3>::bytes));
     TC_SET_SMEM((k_pair_3b4_pr<T, N, kPruneL<N>>), (int)(PrSmem<T, N, kPruneL<N>, 1, 1>::bytes));
@@ -310,7 +317,8 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   // pair densities whose spectra fit the compiled support take the pruned transforms
   constexpr int LP = kPruneL<N>;
   const bool pruned = LP < N && ctx->pair_support <= LP;
-  P.fold = pruned ? 1 : 0;
+  // small boxes run the same kernels on the full support (every box index) otherwise
+  constexpr bool FP = kFullPr<N>;
   // else, when they fit the distributed kernels' support, the cluster-distributed ones
   constexpr int LC = ClPlan<T, N>::L;
   using C0 = ClCfg<T, N, 0>;
@@ -321,11 +329,26 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   const bool dist_chain = dist && CLc > 0 && (ctx->cluster_ok & 1);
   const bool dist_3b4 = dist && CLb > 0 && (ctx->cluster_ok & 2);
   const bool dist_occ = dist && CLo > 0 && (ctx->cluster_ok & 4);
+  P.fold = pruned || FP || dist_chain ? 1 : 0;
   // FP64 pruned kernels run their transforms in fixed point, scaled by the norms of the fields
-  const bool fixed = sizeof(T) == 8 && pruned;
+  const bool fixed = sizeof(T) == 8 && (pruned || FP);
   auto orbital_norms = [&] {
     k_norms<T, N><<<dim3(nj_all, 2), 256, 0, st>>>((cplx<T>*)ctx->d_phi, (cplx<T>*)ctx->d_chi, P.side[0].nket,
                                                    P.side[0].nbra);
+  };
+  // occupied-pair stage on one CTA per item
+  auto launch_occ = [&](const Params<T>& p, int items, int sides) {
+    if constexpr (LP < N) {
+      if (pruned) {
+        k_occ_pairs_pr<T, N, LP><<<dim3(items * p.so, sides), PrCfg<T, N>::threads, OccSmem<T, N, LP>::bytes, st>>>(p);
+        return;
+      }
+    }
+    if constexpr (FP) {
+      k_occ_pairs_pr<T, N, N><<<dim3(items * p.so, sides), PrCfg<T, N>::threads, OccSmem<T, N, N>::bytes, st>>>(p);
+    } else {
+      if (!dist_occ) k_occ_pairs<T, N><<<dim3(items * p.so, sides), TH, p.nsmem * vb, st>>>(p);
+    }
   };
   // 1. orbitals to real space
   stage_mark(ctx, st, 0);
@@ -413,17 +436,12 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
     Pa.nsmem = smem_vols<T, N>(4);
     if (derive_left) Pa.so = ctx->split_occ[0];
     const int q2_items = P.sym ? P.nirr * S.no : S.Nk * S.no;   // irreducible q2 only with symmetry
-    if constexpr (LP < N) {
-      if (pruned)
-        k_occ_pairs_pr<T, N, LP><<<dim3(q2_items * Pa.so, occ_sides), PrCfg<T, N>::threads,
-                                   OccSmem<T, N, LP>::bytes, st>>>(Pa);
-    }
+    launch_occ(Pa, q2_items, occ_sides);
     if constexpr (CLo > 0) {
       if (dist_occ)
         TC_CHECK_CL(launch_cluster(k_occ_pairs_cl<T, N>, dim3(q2_items * Pa.so * CLo, occ_sides), C2::threads,
                                    C2::smem, CLo, st, Pa));
     }
-    if (!pruned && !dist_occ) k_occ_pairs<T, N><<<dim3(q2_items * Pa.so, occ_sides), TH, Pa.nsmem * vb, st>>>(Pa);
     TC_CHECK_LAUNCH("k_occ_pairs");
     if (Pa.so > 1) {
       k_sum_parts<T, N><<<dim3(2 * pw_blocks, occ_sides), 256, 0, st>>>(Pa, 0);
@@ -462,16 +480,12 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
       Pq.side[sd].h3a4 = P.side[sd].bh3a;
       Pq.side[sd].h3b = P.side[sd].bh3b;
     }
-    if constexpr (LP < N) {
-      if (pruned)
-        k_occ_pairs_pr<T, N, LP><<<dim3(Pq.nq2 * Pq.so, 2), PrCfg<T, N>::threads, OccSmem<T, N, LP>::bytes, st>>>(Pq);
-    }
+    launch_occ(Pq, Pq.nq2, 2);
     if constexpr (CLo > 0) {
       if (dist_occ)
         TC_CHECK_CL(launch_cluster(k_occ_pairs_cl<T, N>, dim3(Pq.nq2 * Pq.so * CLo, 2), C2::threads, C2::smem, CLo,
                                    st, Pq));
     }
-    if (!pruned && !dist_occ) k_occ_pairs<T, N><<<dim3(Pq.nq2 * Pq.so, 2), TH, Pq.nsmem * vb, st>>>(Pq);
     TC_CHECK_LAUNCH("k_occ_pairs (band points)");
     if (Pq.so > 1) {
       k_sum_parts<T, N><<<dim3(2 * pw_blocks, 2), 256, 0, st>>>(Pq, 0);
@@ -529,7 +543,13 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
         TC_CHECK_CL(launch_cluster(k_pair_chain_cl<T, N>, dim3(nj_items * P.sc * CLc, nsides), C0::threads,
                                    C0::smem, CLc, st, Pc));
     }
-    if (!pruned && !dist_chain) k_pair_chain<T, N><<<dim3(nj_items * P.sc, nsides), TH, Pc.nsmem * vb, st>>>(Pc);
+    if constexpr (FP) {
+      if (!pruned)
+        k_pair_chain_pr<T, N, N><<<dim3(nj_items * P.sc, nsides), PrCfg<T, N>::threads, PrSmem<T, N, N, 2, 3>::bytes,
+                                   st>>>(Pc);
+    } else {
+      if (!pruned && !dist_chain) k_pair_chain<T, N><<<dim3(nj_items * P.sc, nsides), TH, Pc.nsmem * vb, st>>>(Pc);
+    }
     TC_CHECK_LAUNCH("k_pair_chain");
     stage_mark(ctx, st, 4);
     if (P.sc > 1) {
@@ -562,7 +582,13 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
         TC_CHECK_CL(launch_cluster(k_pair_3b4_cl<T, N>, dim3(nj_items * P.sc * CLb, nsides), C1::threads, C1::smem,
                                    CLb, st, Pb));
     }
-    if (!pruned && !dist_3b4) k_pair_3b4<T, N><<<dim3(nj_items * P.sc, nsides), TH, Pb.nsmem * vb, st>>>(Pb);
+    if constexpr (FP) {
+      if (!pruned)
+        k_pair_3b4_pr<T, N, N><<<dim3(nj_items * P.sc, nsides), PrCfg<T, N>::threads, PrSmem<T, N, N, 1, 1>::bytes,
+                                 st>>>(Pb);
+    } else {
+      if (!pruned && !dist_3b4) k_pair_3b4<T, N><<<dim3(nj_items * P.sc, nsides), TH, Pb.nsmem * vb, st>>>(Pb);
+    }
     TC_CHECK_LAUNCH("k_pair_3b4");
     if (P.sc > 1 && tw[T3B4] != 0) {
       k_sum_parts<T, N><<<dim3(2 * pw_blocks, nsides), 256, 0, st>>>(P, 2);

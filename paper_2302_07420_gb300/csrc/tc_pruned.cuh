@@ -50,11 +50,18 @@ template <int N, int L> struct Sup {
 // cells' spheres at 16^3, 18^3 and 20^3.
 template <int N> constexpr int kPruneL = (N == 16) ? 13 : (N == 18 || N == 20 || N == 24) ? 17 : N;
 
+// Small boxes whose pair densities do not fit that support run these kernels on the full support
+// (L = N): their volumes and spectra fit one CTA's shared memory in FP64 too, and FP64 takes the
+// fixed-point transforms (14-electron gas, FP64 16^3: pair kernels of the full transforms 1.9 ms).
+template <int N> constexpr bool kFullPr = N <= 16;
+
 // Threads per CTA of the pruned kernels: one axis-1 pencil per thread, in FP64 at most 384 threads (a
 // pencil of N double-complex values takes 4 N registers; 12 warps leave 168 each, as 9 would).
 template <typename T, int N> struct PrCfg {
   static constexpr int one = ((N * N + 31) / 32) * 32;
   static constexpr int threads = sizeof(T) == 8 && one > 384 ? 384 : one;
+  // CTAs per SM that the registers are cut for: two of a small FP32 box (16 warps of 128 registers)
+  static constexpr int minb = sizeof(T) == 4 && N <= 16 ? 2 : 1;
 };
 
 // Shared-memory plan: work volume B first; the compact spectra A and C and the three kernel tables
@@ -67,7 +74,10 @@ template <typename T, int N, int L, int NSPEC, int NTAB> struct PrSmem {
   static constexpr size_t bT = (size_t)S::cvol * sizeof(T);
   static constexpr size_t lim = (size_t)kSmemLimit - 1024;
   static constexpr bool spec = bB + NSPEC * bC <= lim;
-  static constexpr bool tab = spec && bB + NSPEC * bC + NTAB * bT <= lim;
+  // (tables only where the CTAs per SM that the launch bounds ask for still fit: 233,472 bytes per SM,
+  // 1 KB of them per CTA reserved; two 16^3 CTAs without tables beat one with, see PrCfg)
+  static constexpr bool tab = spec && bB + NSPEC * bC + NTAB * bT <= lim &&
+                              PrCfg<T, N>::minb * (bB + NSPEC * bC + NTAB * bT + 2048) <= 233472;
   static constexpr size_t bytes = bB + (spec ? NSPEC * bC : 0) + (tab ? NTAB * bT : 0);
 };
 
@@ -233,7 +243,7 @@ template <int N, int L> __device__ __forceinline__ int gidx_c(int c1, int c2, in
 // relation.  Built for FP64; in FP32 the parallel-spin
 // passes' loads dominate and the mirror code is compiled out.
 template <typename T, int N, int L>
-__global__ void __launch_bounds__(PrCfg<T, N>::threads, 1) k_pair_chain_pr(Params<T> P) {
+__global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pair_chain_pr(Params<T> P) {
   using G = Geo<N>;
   using S = Sup<N, L>;
   using SM = PrSmem<T, N, L, 2, 3>;
@@ -256,7 +266,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, 1) k_pair_chain_pr(Param
   const int jocc = kj * P.no + j % P.nb;
   const bool mw = MIR && P.mirror == 1 && j % P.nb < P.no;
   // (the right CTA of output q skipped its pair with j when f_j, in the compute precision, was 0)
-  const bool mr = MIR && P.mirror == 2 && j % P.nb < P.no && (T)(P.occ[j] / P.Nk) != T(0);
+  const bool mr = MIR && P.mirror == 2 && j % P.nb < P.no && weight(P, j) != T(0);
   const int qi_begin = (int)((long long)chunk * M / P.sc), qi_end = (int)((long long)(chunk + 1) * M / P.sc);
   WorkT<T>* B = reinterpret_cast<WorkT<T>*>(smraw);
   cplx<T>* A;
@@ -291,7 +301,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, 1) k_pair_chain_pr(Param
   for (int qi = qi_begin; qi < qi_end; ++qi) {
     const int kq = qi / P.no, mu = qi % P.no;
     const int q = kq * P.nb + mu;
-    const T f = (T)(P.occ[q] / P.Nk);
+    const T f = weight(P, q);
     if (f == T(0)) continue;
     const T ft2ax = f * t2ax;
     const int did = P.delta_id[kj * P.kstride + kq];
@@ -533,7 +543,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, 1) k_pair_chain_pr(Param
 // Pass 2 for 3b4 (Alg. 10), pruned: acc += tw3b4 f ket_q FT^{-1}[-U^pp . FT[-conj(bra_q) w_j]]
 // (same grid and accumulators as k_pair_3b4).
 template <typename T, int N, int L>
-__global__ void __launch_bounds__(PrCfg<T, N>::threads, 1) k_pair_3b4_pr(Params<T> P) {
+__global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pair_3b4_pr(Params<T> P) {
   using G = Geo<N>;
   using S = Sup<N, L>;
   using SM = PrSmem<T, N, L, 1, 1>;
@@ -566,7 +576,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, 1) k_pair_3b4_pr(Params<
   for (int qi = qi_begin; qi < qi_end; ++qi) {
     const int kq = qi / P.no, mu = qi % P.no;
     const int q = kq * P.nb + mu;
-    const T f = (T)(P.occ[q] / P.Nk);
+    const T f = weight(P, q);
     if (f == T(0)) continue;
     const int did = P.delta_id[kj * P.kstride + kq];
     const T* dl = P.delta + did * 3;
@@ -645,7 +655,7 @@ template <typename T, int N, int L> struct OccSmem {
 };
 
 template <typename T, int N, int L>
-__global__ void __launch_bounds__(PrCfg<T, N>::threads, 1) k_occ_pairs_pr(Params<T> P) {
+__global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_occ_pairs_pr(Params<T> P) {
   using G = Geo<N>;
   using S = Sup<N, L>;
   using SM = OccSmem<T, N, L>;
@@ -677,7 +687,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, 1) k_occ_pairs_pr(Params
   cplx<T>* H6 = slice + 4 * (size_t)G::vol;
   auto ridx = [](int i, int a2, int a3) { return SM::w_smem ? G::sidx(i, a2, a3) : G::gidx(i, a2, a3); };
   const size_t NN = G::nn;
-  const T f2 = (T)(P.occ[q2] / P.Nk);
+  const T f2 = weight(P, q2);
   cplx<T>* h3a4 = SD.h3a4 + ((size_t)chunk * P.nq2 + (i2 - P.i2_0)) * 3 * NN;
   cplx<T>* h3b = SD.h3b + ((size_t)chunk * P.nq2 + (i2 - P.i2_0)) * 3 * NN;
   const cplx<T>* bra2 = SD.bra + (size_t)q2 * NN;
@@ -695,7 +705,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, 1) k_occ_pairs_pr(Params
   for (int i1 = i1_begin; i1 < i1_end; ++i1) {
     const int k1 = i1 / P.no, mu1 = i1 % P.no;
     const int q1 = k1 * P.nb + mu1;
-    const T f1 = (T)(P.occ[q1] / P.Nk);
+    const T f1 = weight(P, q1);
     if (f1 == T(0) || f2 == T(0)) continue;
     const int id12 = P.delta_id[k2 * P.kstride + k1];   // Delta = k2 - k1 -> for P(q1,q2)
     const int id21 = P.delta_id[k1 * P.kstride + k2];   // Delta = k1 - k2 -> for P(q2,q1)

@@ -270,6 +270,23 @@ int pick_split(int items, int partners, int sms) {
   return best;
 }
 
+// A launch lasts about waves x pairs per CTA.  The rule above looks at the waves alone and stops at 8
+// chunks, which leaves a small problem at two pairs per CTA on some SMs and none on others; beyond 8 (up
+// to 32, and only up to two waves of CTAs, so that the parts of the accumulators stay few) a count is
+// taken when it saves a tenth of that product (four k-points, three bands, 15^3 FP64 energy: 12 chunks of
+// one pair instead of 8 of one or two).
+int pick_split_small(int items, int partners, int sms) {
+  const int s0 = pick_split(items, partners, sms);
+  auto rounds = [&](int s) {
+    const long long ctas = (long long)items * s;
+    return (ctas + sms - 1) / sms * ((partners + s - 1) / s);
+  };
+  int best = s0;
+  for (int s = 9; s <= std::min(32, partners) && (long long)items * s <= 2ll * sms; ++s)
+    if (10 * rounds(s) <= 9 * rounds(s0) && rounds(s) < rounds(best)) best = s;
+  return best;
+}
+
 int miller_span(const std::vector<std::vector<std::array<int, 3>>>& miller) {
   int span = 0;
   for (int i = 0; i < 3; ++i) {

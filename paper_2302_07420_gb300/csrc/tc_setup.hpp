@@ -76,6 +76,7 @@ bool sphere(const Setup& S, const double kcart[3], std::vector<std::array<int, 3
 // Default partner chunks per CTA item: the s in 1 .. min(8, partners) whose launch of items x s CTAs
 // fills its last wave on `sms` SMs best (a larger s must raise the filled fraction by more than 1 %).
 int pick_split(int items, int partners, int sms);
+int pick_split_small(int items, int partners, int sms);
 // The autotuner's rule over measured times t[1..n]: the smallest s within 2 % of the fastest, so that
 // near-ties go the same way from run to run and fewer chunks (fewer partial sums) win them.
 int smallest_near_best(const double* t, int n);
