@@ -374,7 +374,7 @@ void choose_splits(tc_ctx* c, bool small) {
     sms = 1;
   }
   const Setup& S = c->S;
-  const int M = S.Nk * S.no, nj = c->nj_out;
+  const int M = S.Nk * S.no, nj = c->nj_out / S.nb * (S.nb - c->jb0);
   for (int sides = 1; sides <= 2; ++sides) {
     c->split_occ[sides - 1] = small ? pick_split_small(M * sides, M, sms) : pick_split(M * sides, M, sms);
     c->split_chain[sides - 1] = small ? pick_split_small(nj * sides, M, sms) : pick_split(nj * sides, M, sms);
@@ -424,7 +424,7 @@ void ws_assign(tc_ctx* c, char* base, const WsLayout& L) {
 }
 
 int init_context(const tc_params* params, bool own_workspace, tc_ctx** out, std::string& err, int nkb,
-                 const double* kfrac_band) {
+                 const double* kfrac_band, int jb0) {
   *out = nullptr;
   tc_ctx* c = new (std::nothrow) tc_ctx();
   if (!c) { err = "host allocation failed"; return TC_ERR_OOM; }
@@ -437,6 +437,7 @@ int init_context(const tc_params* params, bool own_workspace, tc_ctx** out, std:
   }
   tc::Setup& S = c->S;
   c->nj_out = (S.nkb > 0 ? S.nkb : S.Nk) * S.nb;
+  c->jb0 = jb0;
   {
     // the left/right conjugation of the occupied-pair fields and the pruned pair-chain transforms
     // both depend on how far the pair-density spectra reach on the box

@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
   const SideArgs<T>& SD = P.side[blockIdx.y];
   const int cid = blockIdx.x / CL;
   const int jitem = cid / P.sc, chunk = cid % P.sc;
-  const int jo = P.sym ? P.irr[jitem / P.nb] * P.nb + jitem % P.nb : jitem, j = P.j0 + jo, kj = j / P.nb;
+  const int jo = out_item(P, jitem), j = P.j0 + jo, kj = j / P.nb;
   const int M = P.Nk * P.no, nj = P.nj_out;
   const int qi_begin = (int)((long long)chunk * M / P.sc), qi_end = (int)((long long)(chunk + 1) * M / P.sc);
   cplx<T>* B = reinterpret_cast<cplx<T>*>(smraw);
@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(ClCfg<T, N, 1>::threads, ClCfg<T, N, 1>::MINB)
   const SideArgs<T>& SD = P.side[blockIdx.y];
   const int cid = blockIdx.x / CL;
   const int jitem = cid / P.sc, chunk = cid % P.sc;
-  const int jo = P.sym ? P.irr[jitem / P.nb] * P.nb + jitem % P.nb : jitem, j = P.j0 + jo, kj = j / P.nb;
+  const int jo = out_item(P, jitem), j = P.j0 + jo, kj = j / P.nb;
   const int M = P.Nk * P.no, nj = P.nj_out;
   const int qi_begin = (int)((long long)chunk * M / P.sc), qi_end = (int)((long long)(chunk + 1) * M / P.sc);
   cplx<T>* B = reinterpret_cast<cplx<T>*>(smraw);

@@ -104,6 +104,7 @@ struct tc_ctx {
   // context (tc_init_band); band h3 chunks; band constants [nkb][4] = (W, Gamma_b) and the band
   // correction scalars [2][nkb][nocc][nbands][kBandScalars] (device)
   int nj_out = 0;
+  int jb0 = 0;                     // bands below jb0 are partners only, not outputs (Davidson's second context)
   int so_band = 1;
   double* d_band = nullptr;
   double2* d_bs = nullptr;
@@ -128,7 +129,7 @@ namespace tc {
 // and -- if own_workspace -- the workspace block.  Returns a tc_status; on
 // failure *out is null and err holds the reason.
 int init_context(const tc_params* p, bool own_workspace, tc_ctx** out, std::string& err, int nkb = 0,
-                 const double* kfrac_band = nullptr);
+                 const double* kfrac_band = nullptr, int jb0 = 0);
 // Complex FP64 scalars per (side, band point, occupied m, output j) of the band corrections:
 // 0 <bra_m|ket_j>, 1-3 <bra_m|grad ket_j>, 4 <bra_m|(W.h1) ket_j>, 5-6 mean(bra_m^* ket_j V2_s),
 // 7-9 mean(ket_j h3b(m)), 10-12 <bra_m|w_j> (w_j including its correction).

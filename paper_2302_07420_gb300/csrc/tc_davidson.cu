@@ -35,7 +35,7 @@ struct DavState {
   double2* w = nullptr;               // [Nk][m][npw_max] kept new vectors, zero rows after the last
   double2* aux_phi = nullptr;         // [Nk][nocc + m][npw_max] partners phi, then w
   double2* aux_chi = nullptr;         // [Nk][nocc + m][npw_max] partners chi, then w
-  double2* hw = nullptr;              // [Nk][nocc + m][npw_max] operator on the aux bands
+  double2* hw = nullptr;              // [Nk][nocc + m][npw_max] operator on the new vectors (partners' rows unused)
   double2* Y = nullptr;               // [Nk][2m][m] right eigenvector coefficients
   double2* Z = nullptr;               // [Nk][2m][m] left eigenvector coefficients
   double2* lam = nullptr;             // [Nk][m] Ritz values, ascending real part
@@ -621,7 +621,7 @@ tc_status ensure_davidson(tc_ctx* c) {
   if (!D) return dav_fail(c, TC_ERR_OOM, "host allocation failed");
   c->dav = D;
   std::string err;
-  const int r = tc::init_context(&p, true, &D->aux, err);
+  const int r = tc::init_context(&p, true, &D->aux, err, 0, nullptr, no);
   if (r != TC_OK) {
     tc::destroy_davidson(c);
     return dav_fail(c, (tc_status)r, "Davidson operator context: " + err);

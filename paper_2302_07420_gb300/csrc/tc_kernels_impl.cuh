@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads, 1) k_pair_chain(Params<T> P) 
   const SideArgs<T>& S = P.side[blockIdx.y];
   // with crystal symmetry only orbitals of irreducible k-points are computed (the rest are unfolded)
   const int jitem = blockIdx.x / P.sc, chunk = blockIdx.x % P.sc;
-  const int jo = P.sym ? P.irr[jitem / P.nb] * P.nb + jitem % P.nb : jitem, j = P.j0 + jo, kj = j / P.nb;
+  const int jo = out_item(P, jitem), j = P.j0 + jo, kj = j / P.nb;
   const int M = P.Nk * P.no, nj = P.nj_out;
   const int qi_begin = (int)((long long)chunk * M / P.sc), qi_end = (int)((long long)(chunk + 1) * M / P.sc);
   cplx<T>* B = vol_slot<T, N>(P, sm, 0, NS);
@@ -812,7 +812,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads, 1) k_pair_3b4(Params<T> P) {
   const SideArgs<T>& S = P.side[blockIdx.y];
   // with crystal symmetry only orbitals of irreducible k-points are computed (the rest are unfolded)
   const int jitem = blockIdx.x / P.sc, chunk = blockIdx.x % P.sc;
-  const int jo = P.sym ? P.irr[jitem / P.nb] * P.nb + jitem % P.nb : jitem, j = P.j0 + jo, kj = j / P.nb;
+  const int jo = out_item(P, jitem), j = P.j0 + jo, kj = j / P.nb;
   const int M = P.Nk * P.no, nj = P.nj_out;
   const int qi_begin = (int)((long long)chunk * M / P.sc), qi_end = (int)((long long)(chunk + 1) * M / P.sc);
   cplx<T>* B = vol_slot<T, N>(P, sm, 0, NS);
@@ -870,12 +870,12 @@ __global__ void __launch_bounds__(Cfg<N>::threads, 1) k_pair_3b4(Params<T> P) {
 // sum_mu ket_mu (alpha + omega v(r)), v = a_pp vu_pp + a_ap vu_ap, without FP64 work per grid point.
 template <typename T, int N> __global__ void k_corr_scalars(Params<T> P) {
   const SideArgs<T>& S = P.side[blockIdx.y];
-  const int nit = P.sym ? P.nirr * P.nb : P.nj_out;
+  const int nit = (P.sym ? P.nirr : P.nj_out / P.nb) * (P.nb - P.jb0);
   const double a0 = 4.0 * 3.14159265358979323846 * P.A[0] / P.Nk, a1 = 4.0 * 3.14159265358979323846 * P.A[1] / P.Nk;
   const double n0x = (double)S.nt[0].x, n0y = (double)S.nt[0].y, cc = P.corr_c[0] + P.corr_c[1];
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nit * P.no; e += gridDim.x * blockDim.x) {
     const int item = e / P.no, mu = e % P.no;
-    const int jo = P.sym ? P.irr[item / P.nb] * P.nb + item % P.nb : item;
+    const int jo = out_item(P, item);
     double* cs = S.cs + ((size_t)jo * P.no + mu) * 6;
     const double fq = P.occ[(P.j0 + jo) / P.nb * P.nb + mu] * P.invOm2;
     cplx<T>* o = reinterpret_cast<cplx<T>*>(cs);
@@ -900,7 +900,7 @@ template <typename T, int N> __global__ void __launch_bounds__(256) k_local(Para
   const SideArgs<T>& S = P.side[blockIdx.z];
   const size_t NN = (size_t)N * N * N;
   const int item = blockIdx.x;
-  const int jo = P.sym ? P.irr[item / P.nb] * P.nb + item % P.nb : item;
+  const int jo = out_item(P, item);
   const int j = P.j0 + jo, kj = j / P.nb;
   const T t2bh1 = P.tw[T2BH1] * S.s2b, t3a3 = P.tw[T3A3], t3b6 = P.tw[T3B6];
   const bool corr = P.div && t3b6 != T(0) && !P.band;
@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(Cfg<N>::threads)
   const SideArgs<T>& S = P.side[side];
   double2* out = side == 0 ? outR : outL;
   if (out == nullptr) return;
-  const int jo = P.sym ? P.irr[blockIdx.x / P.nb] * P.nb + blockIdx.x % P.nb : blockIdx.x;
+  const int jo = out_item(P, blockIdx.x);
   const int kj = (P.j0 + jo) / P.nb;
   const cplx<T>* acc = S.acc + (size_t)jo * G::nn;
   volume3d<T, N, true>(V, [&](int a, int b, int c) { return ldg(acc + G::gidx(a, b, c)); },

@@ -90,6 +90,7 @@ template <typename T, int N> static Params<T> make_params(tc_ctx* ctx, const dou
   P.star_k = ctx->d_star_k;
   P.kstride = S.Nkt;
   P.j0 = 0;
+  P.jb0 = ctx->jb0;
   P.nj_out = S.Nk * S.nb;
   P.i2_0 = 0;
   P.nq2 = S.Nk * S.no;
@@ -517,7 +518,7 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   }
   // 4. pair chains (with symmetry: output orbitals of irreducible k-points only)
   stage_mark(ctx, st, 3);
-  const int nj_items = P.sym ? P.nirr * S.nb : P.nj_out;
+  const int nj_items = (P.sym ? P.nirr : P.nj_out / S.nb) * (S.nb - P.jb0);
   {
     Params<T> Pc = P;
     Pc.nsmem = smem_vols<T, N>(3);

@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pai
   constexpr bool FX = sizeof(T) == 8;
   const SideArgs<T>& SD = P.side[P.side0 + blockIdx.y];
   const int jitem = blockIdx.x / P.sc, chunk = blockIdx.x % P.sc;
-  const int jo = P.sym ? P.irr[jitem / P.nb] * P.nb + jitem % P.nb : jitem, j = P.j0 + jo, kj = j / P.nb;
+  const int jo = out_item(P, jitem), j = P.j0 + jo, kj = j / P.nb;
   const int M = P.Nk * P.no, nj = P.nj_out;
   // mirrored launches (FP64 only: the FP32 kernel is bound by the loads of its parallel-spin
   // passes, which both sides keep, and gains nothing from them): output j as a partner index; write
@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pai
   const SideArgs<T>& SD = P.side[blockIdx.y];
   __shared__ float bbuf[sizeof(T) == 8 ? kBoundBuf : 1];
   const int jitem = blockIdx.x / P.sc, chunk = blockIdx.x % P.sc;
-  const int jo = P.sym ? P.irr[jitem / P.nb] * P.nb + jitem % P.nb : jitem, j = P.j0 + jo, kj = j / P.nb;
+  const int jo = out_item(P, jitem), j = P.j0 + jo, kj = j / P.nb;
   const int M = P.Nk * P.no, nj = P.nj_out;
   const int qi_begin = (int)((long long)chunk * M / P.sc), qi_end = (int)((long long)(chunk + 1) * M / P.sc);
   WorkT<T>* B = reinterpret_cast<WorkT<T>*>(smraw);
