@@ -45,11 +45,11 @@ def build(verbose=False, jobs=None, ptxas_info=False):
     for name in ("tc_noalloc", "tc_batch", "tc_davidson", "tc_symmetry", "tc_peak"):
         steps.append([nvcc] + NVFLAGS + extra + ["-c", os.path.join(SRC, name + ".cu"),
                                                  "-o", os.path.join(BUILD, name + ".o")])
-    for real in REALS:
-        for n in SIZES:
+    for n in SIZES:      # the largest boxes compile longest: they start first
+        for real in REALS:
             obj = os.path.join(BUILD, "tc_inst_%s_%d.o" % (real, n))
-            steps.append([nvcc] + NVFLAGS + extra + ["-DTC_REAL=%s" % real, "-DTC_N=%d" % n, "-c",
-                                                     os.path.join(SRC, "tc_inst.cu"), "-o", obj])
+            steps.insert(0, [nvcc] + NVFLAGS + extra + ["-DTC_REAL=%s" % real, "-DTC_N=%d" % n, "-c",
+                                                        os.path.join(SRC, "tc_inst.cu"), "-o", obj])
     objs = [s[s.index("-o") + 1] for s in steps]
     with cf.ThreadPoolExecutor(max_workers=jobs or os.cpu_count() or 4) as ex:
         logs = list(ex.map(_run, steps))

@@ -229,7 +229,11 @@ __device__ __forceinline__ void cfwd_32(cg::cluster_group& cluster, cplx<T>* B, 
 // Fused pair chains, distributed (same work, accumulators and per-pair arithmetic as
 // k_pair_chain_pr; Algs. 2, 5, 6, 9, 11, 12 and the 2bx terms of Sec. 2.6.3).  Grid
 // (Nk*nb*sc*CL, sides), clusters of CL CTAs along x; cluster = output orbital j and partner chunk.
-template <typename T, int N>
+// ALL as in k_pair_chain_pr, as kernels of their own for FP32 up to 32^3 (kSplitAll); the others hold both
+// forms of the pass (48^3: no faster apart, and minutes of compilation).
+template <typename T, int N> constexpr bool kSplitAll = sizeof(T) == 4 && N <= 32;
+
+template <typename T, int N, bool ALL>
 __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB) k_pair_chain_cl(Params<T> P) {
   using SM = ClCfg<T, N, 0>;
   constexpr int L = SM::L, CL = SM::CL;
@@ -276,9 +280,9 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
   cplx<T>* acc = SD.acc + ((size_t)chunk * nj + jo) * NN;
   cplx<T>* w = SD.w + ((size_t)chunk * nj + jo) * 3 * NN;
   const T* tw = P.tw;
-  const bool need_w = tw[T3A3] != T(0) || tw[T3B4] != T(0);
-  const bool need_z = tw[T2BX1] != T(0) || tw[T3A4] != T(0);
-  const bool need_y = tw[T3B3] != T(0) || tw[T2BX2] != T(0);
+  const bool need_w = ALL || tw[T3A3] != T(0) || tw[T3B4] != T(0);
+  const bool need_z = ALL || tw[T2BX1] != T(0) || tw[T3A4] != T(0);
+  const bool need_y = ALL || tw[T3B3] != T(0) || tw[T2BX2] != T(0);
   const bool need_pp = need_w || need_z || tw[T3B6] != T(0);
   const bool need_F = need_y || tw[T3B5] != T(0) || tw[T3B6] != T(0);
   const bool need_ap = tw[T3B6] != T(0) && !P.no_ap;
@@ -379,7 +383,7 @@ __global__ void __launch_bounds__(ClCfg<T, N, 0>::threads, ClCfg<T, N, 0>::MINB)
             cluster, rb, rank, [&](int, int, int) { return cplx<T>{0, 0}; },
             [&](int, int i2, int i3, cplx<T>(&v)[N]) {
               if (sp == 0) {
-                if (all) {
+                if (ALL || (!kSplitAll<T, N> && all)) {
                   // CH points at a time, their loads issued before any of their reductions
 #pragma unroll
                   for (int c0 = 0; c0 < N; c0 += CH) {

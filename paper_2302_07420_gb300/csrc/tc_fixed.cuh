@@ -18,8 +18,8 @@
 // FP64 transform: against 64-bit results the 3x3x3 apply is off by 1.5e-15 (1.8e-15 in FP64
 // arithmetic), and it takes 222 ms instead of 499; the 2x2x2 gradient 151 instead of 324.  Bounds come from the 2- and max norms of the real-space factors (k_norms;
 // |sum a b| <= |a|_2 |b|_2) and, for spectra, from sums of upper-rounded floats over the spectrum.
-// A bound that is not finite (an infinity or NaN among the inputs) poisons the transform: all
-// its results are NaN, as a floating-point transform of such a volume gives.
+// A bound that is not finite (an infinity or NaN among the inputs, or values beyond 2^900) poisons the
+// transform: all its results are NaN, as a floating-point transform of such a volume gives.
 #pragma once
 #include "tc_kernels.cuh"
 
@@ -42,7 +42,7 @@ template <> struct Scale<double> {
 // Smallest e with b < 2^e (b >= 0), clamped to where every shifted exponent below stays normal.
 __device__ __forceinline__ int fx_exp(double b) {
   const int e = ((__double2hiint(b) >> 20) & 0x7ff) - 1022;
-  return e < -400 ? -400 : e;
+  return e < -900 ? -900 : e;
 }
 constexpr int ceil_log2(long long v) { return v <= 1 ? 0 : 1 + ceil_log2((v + 1) / 2); }
 

@@ -205,12 +205,14 @@ template <typename T, int N> int prepare_kernels(tc_ctx* ctx) {
     TC_SET_SMEM((k_pair_chain<T, N>), (smem_vols<T, N>(3) * vb));
     TC_SET_SMEM((k_pair_3b4<T, N>), (smem_vols<T, N>(2) * vb));
   } else {
-    TC_SET_SMEM((k_pair_chain_pr<T, N, N>), (int)(PrSmem<T, N, N, 2, 3>::bytes));
+    TC_SET_SMEM((k_pair_chain_pr<T, N, N, sizeof(T) == 4>), (int)(PrSmem<T, N, N, 2, 3>::bytes));
+    TC_SET_SMEM((k_pair_chain_pr<T, N, N, false>), (int)(PrSmem<T, N, N, 2, 3>::bytes));
     TC_SET_SMEM((k_pair_3b4_pr<T, N, N>), (int)(PrSmem<T, N, N, 1, 1>::bytes));
     TC_SET_SMEM((k_occ_pairs_pr<T, N, N>), (int)(OccSmem<T, N, N>::bytes));
   }
   if constexpr (kPruneL<N> < N) {
-    TC_SET_SMEM((k_pair_chain_pr<T, N, kPruneL<N>>), (int)(PrSmem<T, N, kPruneL<N>, 2, 3>::bytes));
+    TC_SET_SMEM((k_pair_chain_pr<T, N, kPruneL<N>, sizeof(T) == 4>), (int)(PrSmem<T, N, kPruneL<N>, 2, 3>::bytes));
+    TC_SET_SMEM((k_pair_chain_pr<T, N, kPruneL<N>, false>), (int)(PrSmem<T, N, kPruneL<N>, 2, 3>::bytes));
     TC_SET_SMEM((k_pair_3b4_pr<T, N, kPruneL<N>>), (int)(PrSmem<T, N, kPruneL<N>, 1, 1>::bytes));
     TC_SET_SMEM((k_occ_pairs_pr<T, N, kPruneL<N>>), (int)(OccSmem<T, N, kPruneL<N>>::bytes));
   }
@@ -227,7 +229,10 @@ template <typename T, int N> int prepare_kernels(tc_ctx* ctx) {
   ctx->plan_cl[1] = C1::CL;
   ctx->plan_cl[2] = C2::CL;
   if constexpr (C0::CL > 0)
-    ctx->cluster_ok |= cluster_fits(ctx, k_pair_chain_cl<T, N>, C0::CL, C0::threads, C0::smem) ? 1 : 0;
+    ctx->cluster_ok |= cluster_fits(ctx, k_pair_chain_cl<T, N, kSplitAll<T, N>>, C0::CL, C0::threads, C0::smem) &&
+                               cluster_fits(ctx, k_pair_chain_cl<T, N, false>, C0::CL, C0::threads, C0::smem)
+                           ? 1
+                           : 0;
   if constexpr (C1::CL > 0)
     ctx->cluster_ok |= cluster_fits(ctx, k_pair_3b4_cl<T, N>, C1::CL, C1::threads, C1::smem) ? 2 : 0;
   if constexpr (C2::CL > 0)
@@ -522,6 +527,8 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   {
     Params<T> Pc = P;
     Pc.nsmem = smem_vols<T, N>(3);
+    constexpr bool SA = sizeof(T) == 4;   // FP32: a kernel of its own for launches with every term group on
+    const bool all = all_terms(P);
     if constexpr (LP < N) {
       // two-sided FP64: the right side first, writing the reflections the left side then reads
       const bool mirror = sizeof(T) == 8 && pruned && nsides == 2 && ctx->d_mirror && !P.sym && !band;
@@ -530,24 +537,24 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
         for (int sd = 0; sd < 2; ++sd) {
           Pc.side0 = sd;
           Pc.mirror = 1 + sd;
-          k_pair_chain_pr<T, N, LP><<<dim3(nj_items * P.sc, 1), PrCfg<T, N>::threads,
-                                      PrSmem<T, N, LP, 2, 3>::bytes, st>>>(Pc);
+          (all ? k_pair_chain_pr<T, N, LP, SA> : k_pair_chain_pr<T, N, LP, false>)<<<
+              dim3(nj_items * P.sc, 1), PrCfg<T, N>::threads, PrSmem<T, N, LP, 2, 3>::bytes, st>>>(Pc);
         }
         nl[3] += 1;
       } else if (pruned) {
-        k_pair_chain_pr<T, N, LP><<<dim3(nj_items * P.sc, nsides), PrCfg<T, N>::threads,
-                                    PrSmem<T, N, LP, 2, 3>::bytes, st>>>(Pc);
+        (all ? k_pair_chain_pr<T, N, LP, SA> : k_pair_chain_pr<T, N, LP, false>)<<<
+            dim3(nj_items * P.sc, nsides), PrCfg<T, N>::threads, PrSmem<T, N, LP, 2, 3>::bytes, st>>>(Pc);
       }
     }
     if constexpr (CLc > 0) {
       if (dist_chain)
-        TC_CHECK_CL(launch_cluster(k_pair_chain_cl<T, N>, dim3(nj_items * P.sc * CLc, nsides), C0::threads,
+        TC_CHECK_CL(launch_cluster(all ? k_pair_chain_cl<T, N, kSplitAll<T, N>> : k_pair_chain_cl<T, N, false>, dim3(nj_items * P.sc * CLc, nsides), C0::threads,
                                    C0::smem, CLc, st, Pc));
     }
     if constexpr (FP) {
       if (!pruned)
-        k_pair_chain_pr<T, N, N><<<dim3(nj_items * P.sc, nsides), PrCfg<T, N>::threads, PrSmem<T, N, N, 2, 3>::bytes,
-                                   st>>>(Pc);
+        (all ? k_pair_chain_pr<T, N, N, SA> : k_pair_chain_pr<T, N, N, false>)<<<
+            dim3(nj_items * P.sc, nsides), PrCfg<T, N>::threads, PrSmem<T, N, N, 2, 3>::bytes, st>>>(Pc);
     } else {
       if (!pruned && !dist_chain) k_pair_chain<T, N><<<dim3(nj_items * P.sc, nsides), TH, Pc.nsmem * vb, st>>>(Pc);
     }

@@ -215,6 +215,13 @@ template <int N, int L> __device__ __forceinline__ int gidx_c(int c1, int c2, in
   return (S::box(c1) * N + S::box(c2)) * N + S::box(c3);
 }
 
+// Whether every term group of the pair chains' parallel-spin pass is on (the kernels' ALL).
+template <typename T> inline bool all_terms(const Params<T>& P) {
+  const T* t = P.tw;
+  return (t[T3A3] != T(0) || t[T3B4] != T(0)) && (t[T2BX1] != T(0) || t[T3A4] != T(0)) &&
+         (t[T3B3] != T(0) || t[T2BX2] != T(0)) && t[T3B5] != T(0) && t[T3B6] != T(0);
+}
+
 // Fused pair chains, pruned (same work, grid and accumulators as k_pair_chain):
 //   A  = FT[conj(bra_q) ket_j]                                          on the support
 //   for d: b = FT^{-1}[U^pp_d A];  acc += f Z(q)_d b;  w_d += f ket_q b   (2bx1, 3a4, 3a3's w_j)
@@ -242,7 +249,11 @@ template <int N, int L> __device__ __forceinline__ int gidx_c(int c1, int c2, in
 // and the final transform stay per side: their partner fields (Y, Z, h3b, V) have no such
 // relation.  Built for FP64; in FP32 the parallel-spin
 // passes' loads dominate and the mirror code is compiled out.
-template <typename T, int N, int L>
+// ALL: every term group of the parallel-spin pass is on (all_terms): the pass then has no tests, and the
+// kernel not the other form of it beside it, which alone costs 7 % (4x4x4 FP32: 71.6 against 76.8 ms,
+// by the registers and the order of the loads that the compiler gives the pass).  FP32 only: FP64, bound
+// by its products, gains nothing and keeps both forms in one kernel (ALL = false).
+template <typename T, int N, int L, bool ALL>
 __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pair_chain_pr(Params<T> P) {
   using G = Geo<N>;
   using S = Sup<N, L>;
@@ -284,9 +295,9 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pai
   cplx<T>* acc = SD.acc + ((size_t)chunk * nj + jo) * NN;
   cplx<T>* w = SD.w + ((size_t)chunk * nj + jo) * 3 * NN;
   const T* tw = P.tw;
-  const bool need_w = tw[T3A3] != T(0) || tw[T3B4] != T(0);
-  const bool need_z = tw[T2BX1] != T(0) || tw[T3A4] != T(0);
-  const bool need_y = tw[T3B3] != T(0) || tw[T2BX2] != T(0);
+  const bool need_w = ALL || tw[T3A3] != T(0) || tw[T3B4] != T(0);
+  const bool need_z = ALL || tw[T2BX1] != T(0) || tw[T3A4] != T(0);
+  const bool need_y = ALL || tw[T3B3] != T(0) || tw[T2BX2] != T(0);
   const bool need_pp = need_w || need_z || tw[T3B6] != T(0);
   const bool need_F = need_y || tw[T3B5] != T(0) || tw[T3B6] != T(0);
   const bool need_ap = tw[T3B6] != T(0) && !P.no_ap;
@@ -444,7 +455,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pai
             B, [&](int, int, int) { return cplx<T>{0, 0}; },
             [&](int i2, int i3, cplx<T>(&v)[N]) {
               if (sp == 0) {
-                if (all) {
+                if (ALL || (FX && all)) {
                   auto load = [&](int i) {
                     const int g = G::gidx(i, i2, i3);
                     return Elem{ldg(Zq + d * NN + g),  ldg(ketq + g), ldg(Yj + d * NN + g), ldg(braq + g),
