@@ -300,7 +300,7 @@ def measure_extras(p, c_phi, c_chi, occ, d_phi, d_chi, dev):
     out["davidson_step"] = {"what": "tc_davidson_step: h v, Payne + Gram-Schmidt, h w, FP64 subspace eigenpairs, "
                                     "Ritz vectors + biorthonormalisation (host-synchronous call, wall time)",
                             "ms": 1e3 * td, "subspace_dim": [int(dim.min()), int(dim.max())],
-                            "pair_chains": one_side + (nk * (no + nb)) * (nk * no),
+                            "pair_chains": one_side + (nk * nb) * (nk * no),
                             "lowest_ritz_value_k0": float(eig[0, 0].real)}
     out["symmetric"] = measure_symmetric(p, dev)
     h = synth.WORKLOADS["heg_114"]()
