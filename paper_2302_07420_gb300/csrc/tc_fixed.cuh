@@ -13,11 +13,16 @@
 // is a combination of its inputs with weights of modulus at most 1, taken apart into x +- y at most
 // once (a factor sqrt(2)).  With e_k = ceil(log2 b_k) the magnitudes stay below sqrt(2) 2^62 < 2^63.
 // Values are converted at e_1 and shifted right, rounded, by e_2 - e_1 and e_3 - e_2 before the second
-// and third pass.  The rounding left in a result is about 1.5 units of 2^(e_3 - 62): bt is a few to
-// some tens of times the result's root mean square, so this lies below the 2^-53 sqrt(log2 N) of an
-// FP64 transform: against 64-bit results the 3x3x3 apply is off by 1.5e-15 (1.8e-15 in FP64
-// arithmetic), and it takes 222 ms instead of 499; the 2x2x2 gradient 151 instead of 324.  Bounds come from the 2- and max norms of the real-space factors (k_norms;
-// |sum a b| <= |a|_2 |b|_2) and, for spectra, from sums of upper-rounded floats over the spectrum.
+// and third pass.  Every product and shift is rounded to nearest, so that the errors of a pass add up like
+// independent ones: a result is off by 1 to 26 units of 2^(e_3 - 62) in the root mean square and by up to
+// 120 at the worst point, before its conversion to FP64 (boxes of 9^3 to 24^3, both directions, spectra flat
+// and falling off; on the CPU against long double).  With e_3 from bounds as tight as below, that is 0.1e-16
+// to 2.4e-16 of the results' root mean square and 0.7e-16 to 9e-16 at the worst point; the same codelets in
+// FP64 are off by 1.6e-16 to 3.2e-16 and 6e-16 to 42e-16.  (Values that are the same in every pencil are
+// rounded the same way in every pencil: such a coefficient, where only the two ends of the spheres meet, may
+// be off by N^2 / 2 units.)  Bounds come from the 2- and max norms of the real-space factors (k_norms;
+// |sum a b| <= |a|_2 |b|_2) and, for spectra, from sums of upper-rounded floats over the spectrum; factors
+// that barely overlap in space leave |a|_2 |b|_2, and with it the unit, far above the size of their product.
 // A bound that is not finite (an infinity or NaN among the inputs, or values beyond 2^900) poisons the
 // transform: all its results are NaN, as a floating-point transform of such a volume gives.
 #pragma once
@@ -70,7 +75,12 @@ __device__ __forceinline__ long long to_fx(double v, int k) {
   const int hi = __double2hiint(v), lo = __double2loint(v);
   unsigned long long m = ((unsigned long long)((unsigned)(hi & 0xfffff) | 0x100000u) << 32 | (unsigned)lo) << 11;
   const int t = 1085 - k - ((hi >> 20) & 0x7ff);
-  asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(t));   // twice the magnitude; clamps the shift
+  // twice the magnitude; the instruction clamps the shift
+#ifdef __CUDA_ARCH__
+  asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(t));
+#else
+  m = t < 64 ? m >> t : 0;
+#endif
   const long long r = (long long)((m + 1) >> 1), s = (long long)(hi >> 31);
   return (r ^ s) - s;
 }
@@ -93,16 +103,29 @@ __device__ __forceinline__ cplx<double> from_work(cplx<long long> v, const Scale
   return {from_fx(v.x, s), from_fx(v.y, s)};
 }
 __device__ __forceinline__ cplx<float> from_work(cplx<float> v, const Scale<float>&) { return v; }
-// v / 2^s, rounded
-__device__ __forceinline__ long long fx_shift(long long v, long long half, int s) { return (v + half) >> s; }
-__device__ __forceinline__ cplx<long long> shifted(cplx<long long> v, int s) {
-  const long long half = (1ll << s) >> 1;
-  return {fx_shift(v.x, half, s), fx_shift(v.y, half, s)};
+// v / 2^s to nearest, for the values i of pencil p of a pass.  A half goes up or down by the parity of the
+// bits set in p and in i: always up, shifts by one and two bits would add a quarter and an eighth of a unit to
+// every value.  (To even instead: 15.5 clocks per thread and SM for a 24-point codelet, not 12.6.)
+template <typename T> struct PassShift {
+  __device__ __forceinline__ cplx<T> operator()(cplx<T> v, int) const { return v; }
+};
+template <> struct PassShift<double> {
+  long long add[2];
+  int s;
+  __device__ __forceinline__ cplx<long long> operator()(cplx<long long> v, int i) const {
+    const long long a = add[(i ^ (i >> 1) ^ (i >> 2) ^ (i >> 3) ^ (i >> 4) ^ (i >> 5)) & 1];
+    return {(v.x + a) >> s, (v.y + a) >> s};
+  }
+};
+__device__ __forceinline__ PassShift<double> pass_shift(int s, int p) {
+  const long long up = (1ll << s) >> 1, down = s > 0 ? up - 1 : 0;
+  return (__popc(p) & 1) ? PassShift<double>{{down, up}, s} : PassShift<double>{{up, down}, s};
 }
-__device__ __forceinline__ cplx<long long> pass2(cplx<long long> v, const Scale<double>& s) { return shifted(v, s.s2); }
-__device__ __forceinline__ cplx<long long> pass3(cplx<long long> v, const Scale<double>& s) { return shifted(v, s.s3); }
-__device__ __forceinline__ cplx<float> pass2(cplx<float> v, const Scale<float>&) { return v; }
-__device__ __forceinline__ cplx<float> pass3(cplx<float> v, const Scale<float>&) { return v; }
+// before the second and before the third pass
+__device__ __forceinline__ PassShift<double> pass2(const Scale<double>& s, int p) { return pass_shift(s.s2, p); }
+__device__ __forceinline__ PassShift<double> pass3(const Scale<double>& s, int p) { return pass_shift(s.s3, p); }
+__device__ __forceinline__ PassShift<float> pass2(const Scale<float>&, int) { return {}; }
+__device__ __forceinline__ PassShift<float> pass3(const Scale<float>&, int) { return {}; }
 
 // v 2^-x from above, as a float (x: exponent of a bound on |v|, so that nothing overflows; the
 // conversion rounds up, so that nothing is lost at the other end).
@@ -243,9 +266,9 @@ __device__ __forceinline__ void volume3d(cplx<T>* V, Load load, Emit emit, float
     auto put = [&](int a, int b, int c, cplx<I> v) { W[G::sidx(a, b, c)] = v; };
     fft_pass<I, N, S, A1>([&](int a, int b, int c) { return to_work(V[G::sidx(a, b, c)], sc); }, put);
     __syncthreads();
-    fft_pass<I, N, S, 3>([&](int a, int b, int c) { return pass2(W[G::sidx(a, b, c)], sc); }, put);
+    fft_pass<I, N, S, 3>([&](int a, int b, int c) { return pass2(sc, a * N + b)(W[G::sidx(a, b, c)], c); }, put);
     __syncthreads();
-    fft_pass<I, N, S, A3>([&](int a, int b, int c) { return pass3(W[G::sidx(a, b, c)], sc); },
+    fft_pass<I, N, S, A3>([&](int a, int b, int c) { return FWD ? pass3(sc, a * N + c)(W[G::sidx(a, b, c)], b) : pass3(sc, b * N + c)(W[G::sidx(a, b, c)], a); },
                           [&](int a, int b, int c, cplx<I> v) { emit(a, b, c, from_work(v, sc)); });
   } else if constexpr (FWD) {
     fwd3d<T, N>(V, load, emit);

@@ -170,7 +170,7 @@ template <typename T, int N> int prepare_kernels(tc_ctx* ctx) {
   // twiddles exp(-2 pi i j/L) for every codelet length, FP64 host sin/cos
   static double tw64[2 * kTwTotal];
   static float tw32[2 * kTwTotal];
-  static long long twfx[2 * kTwTotal];   // 2^63 w of the twiddles proper, in long double
+  static long long twfx[2 * kTwTotal];
   for (int i = 0, off = 0; i < kNumTwLens; ++i) {
     const int L = kTwLens[i];
     for (int j = 0; j < L; ++j) {
@@ -179,10 +179,7 @@ template <typename T, int N> int prepare_kernels(tc_ctx* ctx) {
       tw64[2 * (off + j) + 1] = std::sin(a);
       tw32[2 * (off + j)] = (float)std::cos(a);
       tw32[2 * (off + j) + 1] = (float)std::sin(a);
-      const long double al = -2.0L * 3.14159265358979323846264338327950288L * j / L, two63 = 9223372036854775808.0L;
-      const bool quarter = (4 * j) % L == 0;   // 1, -i, -1, i: never loaded
-      twfx[2 * (off + j)] = quarter ? 0 : (long long)std::nearbyint(std::cos(al) * two63);
-      twfx[2 * (off + j) + 1] = quarter ? 0 : (long long)std::nearbyint(std::sin(al) * two63);
+      fx_twiddle(j, L, twfx + 2 * (off + j));
     }
     off += L;
   }

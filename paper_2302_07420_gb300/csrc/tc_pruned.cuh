@@ -120,11 +120,12 @@ __device__ __forceinline__ void pinv_23(WorkT<T>* B, Spec spec, const Scale<T>& 
   __syncthreads();
   for (int p = threadIdx.x; p < L * N; p += blockDim.x) {
     const int c1 = p / N, i2 = p % N;
+    const auto shift = pass2(sc, p);
     W v[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) v[i] = W{0, 0};
 #pragma unroll
-    for (int c3 = 0; c3 < L; ++c3) v[S::box(c3)] = pass2(B[S::bidx(c1, i2, c3)], sc);
+    for (int c3 = 0; c3 < L; ++c3) v[S::box(c3)] = shift(B[S::bidx(c1, i2, c3)], c3);
     Codelet<CT, N, +1>::template run<S::on()>(v);
 #pragma unroll
     for (int i3 = 0; i3 < N; ++i3) B[S::bidx(c1, i2, i3)] = v[i3];
@@ -147,11 +148,12 @@ __device__ __forceinline__ void pass_axis1(WorkT<T>* B, Load load, Body body, bo
     const int i2 = p / N, i3 = p % N;
     cplx<T> v[N];
     if constexpr (FROM_B) {
+      const auto shift = pass3(si, p);
       W u[N];
 #pragma unroll
       for (int i = 0; i < N; ++i) u[i] = W{0, 0};
 #pragma unroll
-      for (int c1 = 0; c1 < L; ++c1) u[S::box(c1)] = pass3(B[S::bidx(c1, i2, i3)], si);
+      for (int c1 = 0; c1 < L; ++c1) u[S::box(c1)] = shift(B[S::bidx(c1, i2, i3)], c1);
       Codelet<CT, N, +1>::template run<S::on()>(u);
 #pragma unroll
       for (int i = 0; i < N; ++i) v[i] = from_work(u[i], si);
@@ -182,9 +184,10 @@ __device__ __forceinline__ void pfwd_32(WorkT<T>* B, Emit emit, const Scale<T>& 
   using CT = decltype(W().x);
   for (int p = threadIdx.x; p < L * N; p += blockDim.x) {
     const int c1 = p / N, i2 = p % N;
+    const auto shift = pass2(sc, p);
     W v[N];
 #pragma unroll
-    for (int i3 = 0; i3 < N; ++i3) v[i3] = pass2(B[S::bidx(c1, i2, i3)], sc);
+    for (int i3 = 0; i3 < N; ++i3) v[i3] = shift(B[S::bidx(c1, i2, i3)], i3);
     Codelet<CT, N, -1>::run(v);
 #pragma unroll
     for (int c3 = 0; c3 < L; ++c3) B[S::bidx(c1, i2, c3)] = v[S::box(c3)];
@@ -192,9 +195,10 @@ __device__ __forceinline__ void pfwd_32(WorkT<T>* B, Emit emit, const Scale<T>& 
   __syncthreads();
   for (int p = threadIdx.x; p < L * L; p += blockDim.x) {
     const int c1 = p / L, c3 = p % L;
+    const auto shift = pass3(sc, p);
     W v[N];
 #pragma unroll
-    for (int i2 = 0; i2 < N; ++i2) v[i2] = pass3(B[S::bidx(c1, i2, c3)], sc);
+    for (int i2 = 0; i2 < N; ++i2) v[i2] = shift(B[S::bidx(c1, i2, c3)], i2);
     Codelet<CT, N, -1>::run(v);
 #pragma unroll
     for (int c2 = 0; c2 < L; ++c2) emit(c1, c2, c3, from_work(v[S::box(c2)], sc));
