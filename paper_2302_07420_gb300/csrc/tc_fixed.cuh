@@ -62,7 +62,7 @@ template <typename T, int LEN> __device__ __forceinline__ Scale<T> fx_scale(doub
     s.k_in = 62 - e1;
     s.s2 = e2 - e1;
     s.s3 = e3 - e2;
-    s.hi_out = (e3 - 62) << 20;
+    s.hi_out = (e3 - 62) * (1 << 20);
     s.poison = (xt < 900 && x0 < 900) ? 0 : 0x7ff80000;   // (fx_exp of an infinity or NaN: 1025)
   }
   return s;
@@ -131,7 +131,7 @@ __device__ __forceinline__ PassShift<float> pass3(const Scale<float>&, int) { re
 // conversion rounds up, so that nothing is lost at the other end).
 __device__ __forceinline__ float fx_float(double v, int x) {
   const int hi = __double2hiint(v) & 0x7fffffff;
-  const int h = hi >= 0x7ff00000 ? hi : (hi > max(0, x << 20) || x < 0) && hi != 0 ? hi - (x << 20) : 0;
+  const int xh = x * (1 << 20), h = hi >= 0x7ff00000 ? hi : (hi > max(0, xh) || x < 0) && hi != 0 ? hi - xh : 0;
   return __double2float_ru(__hiloint2double(h, __double2loint(v)));
 }
 // a 2^x

@@ -65,7 +65,7 @@ template <int N, int L> static void box() {
   std::normal_distribution<double> nd;
   const char* kinds[] = {"flat", "gauss", "exponential"};
   for (int kind = 0; kind < 3; ++kind) {
-    auto weight = [&](double m2) { return kind == 0 ? 1.0 : kind == 1 ? std::exp(-0.2 * m2) : std::exp(-0.5 * std::sqrt(m2)); };
+    auto weight = [&](double m2) { return kind == 0 ? 1.0 : kind == 1 ? std::exp(-0.2 * m2) : 0x1p-60 * std::exp(-0.5 * std::sqrt(m2)); };
     auto random_spectrum = [&](std::vector<cplx<double>>& A, vol& v) {
       A.resize(S::cvol);
       v.assign(G::nn, cl(0));

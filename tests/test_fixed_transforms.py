@@ -18,19 +18,30 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2302_07420_gb300", "csrc")
 
 
-@pytest.fixture(scope="module")
-def lines(tmp_path_factory):
+def _probe(path, *flags):
     gxx = shutil.which("g++")
     if not gxx:
         pytest.skip("g++ not available")
-    exe = str(tmp_path_factory.mktemp("fixed") / "fixed_probe")
-    r = subprocess.run([gxx, "-O2", "-std=c++17", "-w", "-I", os.path.join(ROOT, "tests", "host", "cuda"), "-I", CSRC,
+    exe = str(path / "fixed_probe")
+    r = subprocess.run([gxx, "-std=c++17", "-w", *flags, "-I", os.path.join(ROOT, "tests", "host", "cuda"), "-I", CSRC,
                         "-o", exe, os.path.join(ROOT, "tests", "host", "fixed_probe.cpp")],
                        capture_output=True, text=True)
+    if "-fsanitize=undefined" in flags and "ubsan" in r.stderr:
+        pytest.skip("no sanitizer library")
     assert r.returncode == 0, r.stderr
     out = subprocess.run([exe], capture_output=True, text=True)
     assert out.returncode == 0
-    return [line.split() for line in out.stdout.splitlines()]
+    return out
+
+
+@pytest.fixture(scope="module")
+def lines(tmp_path_factory):
+    return [line.split() for line in _probe(tmp_path_factory.mktemp("fixed"), "-O2").stdout.splitlines()]
+
+
+def test_no_undefined_arithmetic(tmp_path):
+    """No signed overflow and no left shift of a negative value in the transforms and their scales."""
+    assert _probe(tmp_path, "-O1", "-fsanitize=undefined").stderr == ""
 
 
 @pytest.mark.parametrize("direction", ["inv", "fwd"])
