@@ -947,7 +947,8 @@ tc_status tc_energy_grad(tc_ctx* c, const void* phi, const void* chi, const doub
         return cuda_fail(c, e, "derivative tables");
       }
     }
-    const double corr0[2] = {S.corr_c[0], S.corr_c[1]}, amp0[2] = {S.amp[0], S.amp[1]};
+    const double corr0[2] = {S.corr_c[0], S.corr_c[1]}, amp0[2] = {S.amp[0], S.amp[1]},
+                 u_max0[2] = {S.u_max[0], S.u_max[1]};
     double twE[NT];
     term_weights(c, twE, 0.5, 1.0 / 3.0);
     r = TC_OK;
@@ -976,6 +977,7 @@ tc_status tc_energy_grad(tc_ctx* c, const void* phi, const void* chi, const doub
         for (int s = 0; s < 2; ++s) {
           S.corr_c[s] = corr0[s] + a * dk.corr_c[s];
           S.amp[s] = amp0[s] + a * dk.amp[s];
+          S.u_max[s] = u_max0[s] + t * dk.u_max[s];
         }
         r = run_common(c, dphi, dchi, occ, c->d_out_R, nullptr, twE, 1, st, &host_out);
         if (r == TC_OK) r = energy_reduce(c, dphi, dchi, occ, false, true, st, &Epm[sg]);
@@ -987,6 +989,7 @@ tc_status tc_energy_grad(tc_ctx* c, const void* phi, const void* chi, const doub
     for (int s = 0; s < 2; ++s) {
       S.corr_c[s] = corr0[s];
       S.amp[s] = amp0[s];
+      S.u_max[s] = u_max0[s];
     }
     e = c->prec == TC_FP64 ? displace_tables<double>(c, -1, 0.0, st) : displace_tables<float>(c, -1, 0.0, st);
     if (r != TC_OK) return r;

@@ -23,8 +23,10 @@
 // be off by N^2 / 2 units.)  Bounds come from the 2- and max norms of the real-space factors (k_norms;
 // |sum a b| <= |a|_2 |b|_2) and, for spectra, from sums of upper-rounded floats over the spectrum; factors
 // that barely overlap in space leave |a|_2 |b|_2, and with it the unit, far above the size of their product.
-// A bound that is not finite (an infinity or NaN among the inputs, or values beyond 2^900) poisons the
-// transform: all its results are NaN, as a floating-point transform of such a volume gives.
+// Bounds are kept as a scaled value and an exponent until they are whole, so that they hold for values between
+// 2^-950 and 2^1000: results are multiples of at least 2^-1012, and a bound beyond 2^1000 or not finite (an
+// infinity or NaN among the inputs) poisons the transform, all of whose results are then NaN, as a
+// floating-point transform of a volume with such a value gives.
 #pragma once
 #include "tc_kernels.cuh"
 
@@ -44,10 +46,11 @@ template <> struct Scale<double> {
   int poison;      // bits set in the high word of every result: NaN when a bound is not finite
 };
 
-// Smallest e with b < 2^e (b >= 0), clamped to where every shifted exponent below stays normal.
+// Smallest e with b < 2^e (b >= 0; an infinity or NaN: 1025), clamped to where a zero is still shifted out
+// (to_fx) and every result's exponent is that of a normal number (from_fx).
 __device__ __forceinline__ int fx_exp(double b) {
   const int e = ((__double2hiint(b) >> 20) & 0x7ff) - 1022;
-  return e < -900 ? -900 : e;
+  return e < -950 ? -950 : e;
 }
 constexpr int ceil_log2(long long v) { return v <= 1 ? 0 : 1 + ceil_log2((v + 1) / 2); }
 
@@ -63,7 +66,7 @@ template <typename T, int LEN> __device__ __forceinline__ Scale<T> fx_scale(doub
     s.s2 = e2 - e1;
     s.s3 = e3 - e2;
     s.hi_out = (e3 - 62) * (1 << 20);
-    s.poison = (xt < 900 && x0 < 900) ? 0 : 0x7ff80000;   // (fx_exp of an infinity or NaN: 1025)
+    s.poison = (xt < 1000 && x0 < 1000) ? 0 : 0x7ff80000;
   }
   return s;
 }
@@ -134,9 +137,10 @@ __device__ __forceinline__ float fx_float(double v, int x) {
   const int xh = x * (1 << 20), h = hi >= 0x7ff00000 ? hi : (hi > max(0, xh) || x < 0) && hi != 0 ? hi - xh : 0;
   return __double2float_ru(__hiloint2double(h, __double2loint(v)));
 }
-// a 2^x
-__device__ __forceinline__ double fx_unscale(float a, int x) {
-  return x >= 1000 ? __hiloint2double(0x7ff00000, 0) : (double)a * __hiloint2double((x + 1023) << 20, 0);
+// a 2^x for |x| <= 2000, in two steps
+__device__ __forceinline__ double fx_unscale(double a, int x) {
+  const int h = x / 2;
+  return a * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((x - h + 1023) << 20, 0);
 }
 
 // Bounds of a spectrum: the largest modulus and the sum of the moduli of the values added, in floats
@@ -146,7 +150,7 @@ struct SpecBound {
   // |v| w, w >= 0 from above
   __device__ __forceinline__ void add(cplx<double> v, float w, int x) {
     const float a = __fmul_ru(__fadd_ru(fx_float(v.x, x), fx_float(v.y, x)), w);
-    m = (a <= m) ? m : a;   // a NaN is kept
+    m = (a <= m) ? m : a;   // (a NaN stays in the sum)
     s = __fadd_ru(s, a);
   }
 };
@@ -214,7 +218,7 @@ __device__ __forceinline__ Scale<T> spectrum_scale(int n, Value value, float* bu
   }
 }
 
-// |u p| from above at compact index (c1, c2, c3), u a kernel-table value
+// |u p| 2^-x from above at compact index (c1, c2, c3), u a kernel-table value, 2^x a bound on its table
 struct PBound {
   float c[3], b[3][3], slop;
 };
@@ -235,14 +239,14 @@ template <typename T> __device__ __forceinline__ PBound pbound_setup(const Param
   q.slop *= 1e-6f;   // float rounding of the components, against cancellation at small |p|
   return q;
 }
-__device__ __forceinline__ float pbound(const PBound& q, double u, float m1, float m2, float m3) {
+__device__ __forceinline__ float pbound(const PBound& q, double u, int x, float m1, float m2, float m3) {
   float p2 = 0.f;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const float p = q.c[d] + m1 * q.b[0][d] + m2 * q.b[1][d] + m3 * q.b[2][d];
     p2 = fmaf(p, p, p2);
   }
-  return __fmul_ru(__double2float_ru(fabs(u)), sqrtf(p2) * 1.00001f + q.slop);
+  return __fmul_ru(fx_float(u, x), sqrtf(p2) * 1.00001f + q.slop);
 }
 
 // 3D transforms of one volume per CTA (fwd3d, inv3d of tc_fft.cuh; same arguments) in fixed point where
@@ -278,34 +282,46 @@ __device__ __forceinline__ void volume3d(cplx<T>* V, Load load, Emit emit, float
 }
 
 // Norms of the volumes a[v], v < count (blockIdx.x), into out: the 2-norm over the grid points and the
-// largest modulus (its components added, so both from above up to rounding).
-template <typename T, int N> __global__ void __launch_bounds__(256) k_norms(const cplx<T>* a, const cplx<T>* b, Norm* na, Norm* nb) {
-  const cplx<T>* v = (blockIdx.y == 0 ? a : b) + (size_t)blockIdx.x * N * N * N;
-  Norm* out = (blockIdx.y == 0 ? na : nb) + blockIdx.x;
-  double s = 0.0, m = 0.0;
-  for (int r = threadIdx.x; r < N * N * N; r += blockDim.x) {
-    const double t = fabs((double)v[r].x) + fabs((double)v[r].y);
-    s = fma(t, t, s);
-    m = (t <= m) ? m : t;
+// largest modulus, from above (parts in 10^6).  The largest component's exponent first: the squares are of values
+// scaled by it, which neither overflow nor vanish (2-norms from squares as they are: infinite from 2^512, 0
+// below 2^-538).  The scaled values are floats made of the upper word, as the FP64 pipe would take 27 us for a
+// 24^3 volume; the words stay in registers between the two (27 points per thread at 24^3).
+template <int N> __global__ void __launch_bounds__(512) k_norms(const cplx<double>* a, const cplx<double>* b, Norm* na, Norm* nb) {
+  constexpr int W = 512 / 32, M = (N * N * N + 511) / 512;
+  const cplx<double>* v = (blockIdx.y == 0 ? a : b) + (size_t)blockIdx.x * N * N * N;
+  __shared__ float ss[W];
+  __shared__ int sh[W];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int u[2 * M], h = 0;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const int r = threadIdx.x + 512 * i;
+    const cplx<double> t = r < N * N * N ? v[r] : cplx<double>{0, 0};
+    u[2 * i] = __double2hiint(t.x) & 0x7fffffff;
+    u[2 * i + 1] = __double2hiint(t.y) & 0x7fffffff;
   }
-  __shared__ double ss[8], sm[8];
-  for (int o = 16; o > 0; o >>= 1) {
-    s += __shfl_xor_sync(0xffffffffu, s, o);
-    const double t = __shfl_xor_sync(0xffffffffu, m, o);
-    m = (t <= m) ? m : t;
+#pragma unroll
+  for (int i = 0; i < 2 * M; ++i) h = max(h, u[i]);
+  h = __reduce_max_sync(0xffffffffu, h);
+  if (lane == 0) sh[wid] = h;
+  __syncthreads();
+  for (int w = 0; w < W; ++w) h = max(h, sh[w]);
+  const int x = (h >> 20) - 1023, shift = (896 + x) * (1 << 20);   // the largest in [1, 2), exponent field 127
+  float s = 0.f;
+#pragma unroll
+  for (int i = 0; i < 2 * M; ++i) {
+    const float f = __int_as_float(max(0, u[i] + 1 - shift) << 3);
+    s = __fmaf_ru(f, f, s);
   }
-  if ((threadIdx.x & 31) == 0) {
-    ss[threadIdx.x >> 5] = s;
-    sm[threadIdx.x >> 5] = m;
-  }
+  for (int o = 16; o > 0; o >>= 1) s = __fadd_ru(s, __shfl_xor_sync(0xffffffffu, s, o));
+  if (lane == 0) ss[wid] = s;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) {
-      s += ss[w];
-      m = (sm[w] <= m) ? m : sm[w];
-    }
-    out->two = sqrt(s);
-    out->inf = m;
+    for (int w = 1; w < W; ++w) s = __fadd_ru(s, ss[w]);
+    const double inf = __hiloint2double(0x7ff00000, 0);   // (an infinity or NaN among the values)
+    Norm n = {h < 0x7ff00000 ? fx_unscale(sqrt((double)s), x) : inf,
+              h < 0x7ff00000 ? fx_unscale(1.4143 * __hiloint2double((h & 0xfffff) + 1 + 0x3ff00000, 0), x) : inf};
+    (blockIdx.y == 0 ? na : nb)[blockIdx.x] = n;
   }
 }
 

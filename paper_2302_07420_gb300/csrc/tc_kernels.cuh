@@ -92,6 +92,7 @@ template <typename T> struct Params {
   int i2_0, nq2;         // occupied-pair stage: q2 items i2_0 .. i2_0 + nq2 - 1 (item = k no + mu)
   int h3_only;           // occupied-pair stage: the two h3 kinds only (parallel spins, no h6)
   int no_ap;             // pair stages without the work that reads only the antiparallel kernel table
+  int u_exp[2];          // values of tabU below 2^u_exp in modulus, per channel (fixed-point transforms' bounds)
   int fold;              // the pruned pair chains run: Z carries f_q, Y and tn are over tw3b5 (if not 0)
   int band;              // outputs at band points: no SCF-mesh 3b6 corrections in k_finalize
   int nkb;               // band points (band contexts)

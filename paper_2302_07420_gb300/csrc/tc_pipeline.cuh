@@ -96,6 +96,8 @@ template <typename T, int N> static Params<T> make_params(tc_ctx* ctx, const dou
   P.nq2 = S.Nk * S.no;
   P.h3_only = 0;
   P.no_ap = ctx->skip_ap;
+  for (int s = 0; s < 2; ++s)
+    P.u_exp[s] = S.u_max[s] > 0 ? std::min(std::max(std::ilogb(S.u_max[s]) + 1, -950), 1023) : -950;
   P.band = 0;
   P.nkb = S.nkb;
   P.bandc = ctx->d_band;
@@ -334,10 +336,14 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
   const bool dist_occ = dist && CLo > 0 && (ctx->cluster_ok & 4);
   P.fold = pruned || FP || dist_chain ? 1 : 0;
   // FP64 pruned kernels run their transforms in fixed point, scaled by the norms of the fields
-  const bool fixed = sizeof(T) == 8 && (pruned || FP);
+  constexpr bool FX = sizeof(T) == 8 && (LP < N || FP);
+  const bool fixed = FX && (pruned || FP);
+  // norms of count volumes at a and, if given, as many at b
+  auto norms = [&](int count, const cplx<T>* a, Norm* na, const cplx<T>* b = nullptr, Norm* nb = nullptr) {
+    if constexpr (FX) k_norms<N><<<dim3(count, b ? 2 : 1), 512, 0, st>>>(a, b, na, nb);
+  };
   auto orbital_norms = [&] {
-    k_norms<T, N><<<dim3(nj_all, 2), 256, 0, st>>>((cplx<T>*)ctx->d_phi, (cplx<T>*)ctx->d_chi, P.side[0].nket,
-                                                   P.side[0].nbra);
+    norms(nj_all, (cplx<T>*)ctx->d_phi, P.side[0].nket, (cplx<T>*)ctx->d_chi, P.side[0].nbra);
   };
   // occupied-pair stage on one CTA per item
   auto launch_occ = [&](const Params<T>& p, int items, int sides) {
@@ -511,9 +517,9 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
     // tw3b6 n and, contiguous per side where they were written, Y and h3b (part 0)
     for (int sd = 0; sd < nsides; ++sd) {
       const SideArgs<T>& D = P.side[sd];
-      k_norms<T, N><<<dim3(1, 1), 256, 0, st>>>(D.tn, D.tn, D.nn, D.nn);
-      k_norms<T, N><<<dim3(P.nj_out * 3, 1), 256, 0, st>>>(D.Y, D.Y, D.nY, D.nY);
-      k_norms<T, N><<<dim3(S.Nk * S.no * 3, 1), 256, 0, st>>>(D.h3b, D.h3b, D.nh3b, D.nh3b);
+      norms(1, D.tn, D.nn);
+      norms(P.nj_out * 3, D.Y, D.nY);
+      norms(S.Nk * S.no * 3, D.h3b, D.nh3b);
     }
     TC_CHECK_LAUNCH("k_norms");
     nl[2] += 3 * nsides;
@@ -570,8 +576,7 @@ int run_pipeline(tc_ctx* ctx, const double2* cphi, const double2* cchi, double2*
       nl[4] += 2;
     }
     if (fixed && tw[T3B4] != 0) {
-      for (int sd = 0; sd < nsides; ++sd)
-        k_norms<T, N><<<dim3(P.nj_out * 3, 1), 256, 0, st>>>(P.side[sd].w, P.side[sd].w, P.side[sd].nw, P.side[sd].nw);
+      for (int sd = 0; sd < nsides; ++sd) norms(P.nj_out * 3, P.side[sd].w, P.side[sd].nw);
       TC_CHECK_LAUNCH("k_norms");
       nl[4] += nsides;
     }

@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pai
     SpecBound sb[2];
     double b_inf[2] = {0, 0}, b_two[2] = {0, 0};   // max norm and 2-norm of FT^{-1}[U_d A] on the grid
     PBound pb;
-    int xa = 0;
+    int xa = 0;   // |A| < 2^xa; the bounds of u_s |p| A are in units of 2^(xa + P.u_exp[s])
     if constexpr (FX) {
       const double two = SD.nket[j].two * SD.nbra[q].two;
       s_rho = fx_scale<T, N>(SD.nket[j].inf * SD.nbra[q].inf, two);
@@ -367,8 +367,8 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pai
       if constexpr (FX) {
         const int g = gidx_c<N, L>(c1, c2, c3);
         const float m1 = S::mil(c1), m2 = S::mil(c2), m3 = S::mil(c3);
-        sb[0].add(a, pbound(pb, __ldg(Upp + g), m1, m2, m3), xa);
-        if (need_ap) sb[1].add(a, pbound(pb, __ldg(Uap + g), m1, m2, m3), xa);
+        sb[0].add(a, pbound(pb, __ldg(Upp + g), P.u_exp[0], m1, m2, m3), xa);
+        if (need_ap) sb[1].add(a, pbound(pb, __ldg(Uap + g), P.u_exp[1], m1, m2, m3), xa);
       }
     };
     if (mr) {
@@ -394,10 +394,11 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_pai
       block_bounds<2>(sb, bbuf);
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
-        b_inf[s] = fx_unscale(sb[s].s, xa);
-        const double m = fx_unscale(sb[s].m, xa);
-        b_two[s] = sqrt((double)G::nn * m * b_inf[s]);   // N sum |x|^2 <= N max|x| sum|x|
-        s_inv[s] = fx_scale<T, L>(m, b_inf[s]);
+        const double m = sb[s].m, t = sb[s].s;
+        const int xb = xa + P.u_exp[s];
+        b_inf[s] = fx_unscale(t, xb);
+        b_two[s] = fx_unscale(sqrt((double)G::nn * m * t), xb);   // N sum |x|^2 <= N max|x| sum|x|
+        s_inv[s] = fx_scale<T, L>(fx_unscale(m, xb), b_inf[s]);
       }
     }
     if (P.div && kq == kj && t3b6 != T(0)) {
@@ -750,7 +751,7 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_occ
         const T* U = P.tabU + ((size_t)(which ? id12 : id21) * 2) * NN;
 #pragma unroll
         for (int s = 0; s < 2; ++s)
-          (which ? sb[2 + s] : sb[s]).add(a, pbound(which ? pb2 : pb1, __ldg(U + s * NN + g), m1, m2, m3), which ? x2 : x1);
+          (which ? sb[2 + s] : sb[s]).add(a, pbound(which ? pb2 : pb1, __ldg(U + s * NN + g), P.u_exp[s], m1, m2, m3), which ? x2 : x1);
       }
     };
     pass_axis1<T, N, L, false>(
@@ -775,7 +776,8 @@ __global__ void __launch_bounds__(PrCfg<T, N>::threads, PrCfg<T, N>::minb) k_occ
       for (int i = 0; i < 4; ++i)
       {
         const double fi = i < 2 ? 1.0 : i == 2 ? (double)f1 : 2.0 * (double)f1;
-        s_inv[i] = fx_scale<T, L>(fi * fx_unscale(sb[i].m, i < 2 ? x1 : x2), fi * fx_unscale(sb[i].s, i < 2 ? x1 : x2));
+        const int x = (i < 2 ? x1 : x2) + P.u_exp[i & 1];
+        s_inv[i] = fx_scale<T, L>(fx_unscale(fi * sb[i].m, x), fx_unscale(fi * sb[i].s, x));
       }
     }
     // 3a2 correction pieces for pairs at the same k (Eqs. divcor_3a2_*_density_matrix_mixing)

@@ -418,6 +418,7 @@ static void value_tables(Setup& S) {
   for (int s = 0; s < 2; ++s) {
     S.corr_c[s] = kd.corr_c[s];
     S.amp[s] = kd.amp[s];
+    S.u_max[s] = kd.u_max[s];
   }
 }
 
@@ -508,6 +509,7 @@ void kernel_data(const Setup& S, int mode, KernelData& kd) {
   for (int s = 0; s < 2; ++s) {
     kd.corr_c[s] = ch_corr(ch[s], S.Gamma0, p.ushort_factor, S.Nk);
     kd.amp[s] = ch_amp(ch[s]);
+    kd.u_max[s] = 0.0;
   }
   // exchange tables at p = Delta + G; V uses the parallel-spin channel
   kd.tabV.assign((size_t)S.ndelta * 2 * N, 0.0);
@@ -535,6 +537,7 @@ void kernel_data(const Setup& S, int mode, KernelData& kd) {
             V[N + g] = (coul * k4Pi / p2 - lap - gsq) / S.Omega;
             U[g] = ch_u(p2, ch[0]) / S.Omega;
             U[N + g] = ch_u(p2, ch[1]) / S.Omega;
+            for (int s = 0; s < 2; ++s) kd.u_max[s] = std::max(kd.u_max[s], std::fabs(U[s * N + g]));
           }
         }
   // Hartree-type tables at G (G = 0 dropped), both channels summed

@@ -38,6 +38,7 @@ struct Setup {
   std::vector<double> hartV;   // [2][N]          (V_pp + V_ap)(G) right / left, 0 at G = 0
   std::vector<double> hartU;   // [N]             (u~pp + u~ap)(G), 0 at G = 0
   std::vector<double> hartUs;  // [2][N]          u~_s(G) (NOT divided by Omega), 0 at G = 0
+  double u_max[2]{};           // largest |u~_s| of tabU, s = pp, ap
   double corr_c[2]{};          // (4 pi A_s)^2 Gamma0 + x 4 pi A_s u_short,s / Nk
   double amp[2]{};             // A_s as used by the corrections (4 pi A_s / Nk)
 };
@@ -48,7 +49,7 @@ struct Setup {
 // Coulomb part).
 struct KernelData {
   std::vector<double> tabV, tabU, hartV, hartU, hartUs;
-  double corr_c[2]{}, amp[2]{};
+  double corr_c[2]{}, amp[2]{}, u_max[2]{};
 };
 enum { KD_VALUE = -1, KD_DA_PP = 0, KD_DA_AP = 1, KD_DC_PP = 2, KD_DC_AP = 3 };
 void kernel_data(const Setup& S, int mode, KernelData& kd);

@@ -53,6 +53,12 @@ inline float __double2float_ru(double v) {
 // (sums and products of two floats are exact, or rounded once below float's half unit, in double)
 inline float __fadd_ru(float a, float b) { return __double2float_ru((double)a + b); }
 inline float __fmul_ru(float a, float b) { return __double2float_ru((double)a * b); }
+inline float __fmaf_ru(float a, float b, float c) { return __double2float_ru((double)a * b + c); }
+inline float __int_as_float(int i) {
+  float f;
+  std::memcpy(&f, &i, 4);
+  return f;
+}
 inline void __syncthreads() {}
 inline void __threadfence() {}
 inline void sincospi(double x, double* s, double* c) {
