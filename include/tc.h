@@ -264,8 +264,9 @@ tc_status tc_fft3d(int n, int precision, int sign, void* data, int batch, void* 
 enum { TC_NSTAGES = 6 };
 tc_status tc_profile(tc_ctx* ctx, int enable);
 /* Autotuner of the partner-chunk counts: runs the operator on the given
- * inputs once per candidate count s = 1 .. min(8, Nk nocc) (after one
- * warm-up), for two-sided launches (tc_apply, tc_energy_grad) and then for
+ * inputs once per candidate count s = 1 .. min(8, Nk nocc) and once at
+ * tc_init's counts where those are larger (small problems: up to 32; after
+ * one warm-up), for two-sided launches (tc_apply, tc_energy_grad) and then for
  * one-sided ones (tc_energy, tc_davidson_step), and keeps, separately for
  * each, the smallest s whose device time is within 2 % of the shortest for
  * the occupied-pair stage and for the pair-chain and 3b4 stages; so_out /

@@ -1139,6 +1139,10 @@ tc_status tc_autotune(tc_ctx* c, const void* phi, const void* chi, const double*
   const int M = S.Nk * S.no;
   const int smax = std::min(8, M);
   const bool prof_was = c->profile;
+  int so[2] = {c->split_occ[0], c->split_occ[1]}, sc[2] = {c->split_chain[0], c->split_chain[1]};
+  // candidates 1 .. smax and, last, the default counts where those are larger (small problems: up to 32)
+  tc::choose_splits(c);
+  const int so_def[2] = {c->split_occ[0], c->split_occ[1]}, sc_def[2] = {c->split_chain[0], c->split_chain[1]};
   // workspace for the largest candidate
   c->so_max = std::max(c->so_max, smax);
   c->sc_max = std::max(c->sc_max, smax);
@@ -1149,15 +1153,15 @@ tc_status tc_autotune(tc_ctx* c, const void* phi, const void* chi, const double*
   double tw[NT];
   term_weights(c, tw, 1.0, 1.0);
   bool host_out = false;
-  int so[2] = {c->split_occ[0], c->split_occ[1]}, sc[2] = {c->split_chain[0], c->split_chain[1]};
   // two-sided launches (tc_apply, tc_energy_grad), then one-sided ones (tc_energy, tc_davidson_step)
   for (int nsides = 2; nsides >= 1 && rs == TC_OK; --nsides) {
-    double t_occ[9] = {}, t_chain[9] = {};
-    for (int s = 0; s <= smax; ++s) {
+    double t_occ[10] = {}, t_chain[10] = {};
+    const int o_def = so_def[nsides - 1], c_def = sc_def[nsides - 1];
+    const int n_occ = smax + (o_def > smax), n_chain = smax + (c_def > smax);
+    for (int s = 0; s <= std::max(n_occ, n_chain); ++s) {
       // s = 0 is an untimed warm-up with one chunk; then one measured apply per candidate
-      const int cand = s == 0 ? 1 : s;
-      c->split_occ[nsides - 1] = cand;
-      c->split_chain[nsides - 1] = cand;
+      c->split_occ[nsides - 1] = s > smax ? o_def : std::max(s, 1);
+      c->split_chain[nsides - 1] = s > smax ? c_def : std::max(s, 1);
       for (int i = 0; i < 8; ++i) c->stage_ms[i] = 0.0;
       rs = run_common(c, phi, chi, occ, c->d_out_R, nsides == 2 ? c->d_out_L : nullptr, tw, nsides, st, &host_out);
       if (rs != TC_OK) break;
@@ -1166,8 +1170,9 @@ tc_status tc_autotune(tc_ctx* c, const void* phi, const void* chi, const double*
       t_chain[s] = c->stage_ms[3] + c->stage_ms[4];
     }
     if (rs != TC_OK) break;
-    so[nsides - 1] = tc::smallest_near_best(t_occ, smax);
-    sc[nsides - 1] = tc::smallest_near_best(t_chain, smax);
+    const int bo = tc::smallest_near_best(t_occ, n_occ), bc = tc::smallest_near_best(t_chain, n_chain);
+    so[nsides - 1] = bo > smax ? o_def : bo;
+    sc[nsides - 1] = bc > smax ? c_def : bc;
   }
   tc_profile(c, prof_was ? 1 : 0);
   c->split_occ[0] = so[0];
