@@ -44,6 +44,8 @@
  * kernel as one the device cannot hold (as cudaOccupancyMaxActiveClusters
  * reporting 0 would): its contexts run the one-CTA kernels with full
  * transforms instead (tc_pair_kernels reports it; results equal to rounding).
+ * TC_FAULT=nochunks makes tc_init and tc_init_batch treat the workspace for
+ * more than 8 partner chunks (small problems) as too large: at most 8 then.
  * TC_ERR_TIMEOUT is otherwise not returned: no kernel of this library waits
  * on a flag or on another kernel.
  * Threads: a context is not thread-safe; distinct contexts are independent.

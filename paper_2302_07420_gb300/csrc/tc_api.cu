@@ -366,8 +366,9 @@ size_t side_field_vols(int Nk, int nb, int no, int so_max, int sc_max, int nj_ou
 // Number of partner chunks s for a launch of `items` CTA items (per chunk one CTA): the s
 // (1 <= s <= min(8, partners)) that fills the last wave of CTAs over the SMs best, the
 // smallest such s when several are within 1 %.  small: more chunks where so few items leave SMs idle
-// (pick_split_small).
+// (pick_split_small), unless their parts would take too much memory (few_chunks).
 void choose_splits(tc_ctx* c, bool small) {
+  small = small && !c->few_chunks;
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || sms <= 0) {
     cudaGetLastError();
@@ -504,7 +505,16 @@ int init_context(const tc_params* params, bool own_workspace, tc_ctx** out, std:
   }
   // workspace: real-space fields, per-side fields, correction scalars, scratch (zeroed once)
   if (own_workspace) {
-    const WsLayout L = ws_layout(c);
+    WsLayout L = ws_layout(c);
+    // the finer chunks of small problems multiply the parts of the accumulators by up to 4: only where
+    // that leaves the memory to others (a sixteenth of what is free)
+    size_t fr = 0, tot = 0;
+    if (e == cudaSuccess) ok(cudaMemGetInfo(&fr, &tot));
+    if (L.total > fr / 16 || injected_fault("chunks") != TC_OK) {
+      c->few_chunks = true;
+      choose_splits(c);
+      L = ws_layout(c);
+    }
     if (e == cudaSuccess) ok(cudaMalloc(&c->d_ws, L.total));
     if (e == cudaSuccess) ok(cudaMemset(c->d_ws, 0, L.total));
     if (e == cudaSuccess) ws_assign(c, static_cast<char*>(c->d_ws), L);
@@ -622,6 +632,7 @@ int injected_fault(const char* site) {
   if (at == "launch" && f == "timeout") return TC_ERR_TIMEOUT;
   if (at == "cluster" && f == "nocluster") return TC_ERR_UNSUPPORTED;
   if (at == "mirror" && f == "nomirror") return TC_ERR_OOM;
+  if (at == "chunks" && f == "nochunks") return TC_ERR_OOM;
   return TC_OK;
 }
 

@@ -175,8 +175,6 @@ tc_status tc_init_batch(int ncell, const tc_params* params, tc_ctx** out) {
     if (r != TC_OK) return bail((tc_status)r, "cell " + std::to_string(i) + ": " + err);
     cell->batch_owner = true;
     B->cells.push_back(cell);
-    B->layouts.push_back(tc::ws_layout(cell));
-    B->lane_bytes = std::max(B->lane_bytes, B->layouts.back().total);
     const tc::Setup& S = cell->S;
     const double pairs = 4.0 * (double)S.Nk * S.nb * (double)S.Nk * S.no;
     B->cost.push_back(pairs * (double)S.N * std::log2((double)S.N));
@@ -185,7 +183,24 @@ tc_status tc_init_batch(int ncell, const tc_params* params, tc_ctx** out) {
   cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
   if (e != cudaSuccess) return bail(TC_ERR_CUDA, cudaGetErrorString(e));
   const size_t budget = free_b / 4;   // at most a quarter of the free memory for the lanes
-  B->lanes_max = (int)std::min<size_t>({(size_t)tc::kMaxLanes, (size_t)ncell, std::max<size_t>(1, budget / B->lane_bytes)});
+  const size_t want = std::min<size_t>(tc::kMaxLanes, ncell);
+  auto chunks = [](tc_ctx* cell, bool few) {
+    cell->few_chunks = few;
+    tc::choose_splits(cell);
+    return tc::ws_layout(cell);
+  };
+  // the finer chunks of small cells only where they cost no lane: within the largest cell's workspace
+  // without them, or within the budget of every lane
+  size_t room = budget / want;
+  for (tc_ctx* cell : B->cells) room = std::max(room, chunks(cell, true).total);
+  const bool few = tc::injected_fault("chunks") != TC_OK;
+  for (tc_ctx* cell : B->cells) {
+    B->layouts.push_back(chunks(cell, few));
+    if (B->layouts.back().total > room) B->layouts.back() = chunks(cell, true);
+    B->lane_bytes = std::max(B->lane_bytes, B->layouts.back().total);
+  }
+  const size_t fit = budget / B->lane_bytes;
+  B->lanes_max = (int)std::min(want, std::max<size_t>(1, fit));
   e = cudaMalloc((void**)&B->d_ws, (size_t)B->lanes_max * B->lane_bytes);
   if (e != cudaSuccess) return bail(e == cudaErrorMemoryAllocation ? TC_ERR_OOM : TC_ERR_CUDA, cudaGetErrorString(e));
   // zeroed once: every later read of the workspace follows a write of the same cell

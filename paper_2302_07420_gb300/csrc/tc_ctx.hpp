@@ -52,6 +52,7 @@ struct tc_ctx {
   // launches (chosen from the SM count, see choose_splits) and the largest of each
   int split_occ[2] = {1, 1}, split_chain[2] = {1, 1};
   int so_max = 1, sc_max = 1;
+  bool few_chunks = false;         // at most 8 chunks: the finer ones' workspace is too large for this device
   // workspace block holding d_phi .. d_scratch (owned unless the context belongs to a batch)
   void* d_ws = nullptr;
   bool ws_owned = true;

@@ -2,7 +2,8 @@
 
 Twelve occupied states on a 15^3 box: tc_init gives the occupied-pair stage 12 chunks of one pair.  Eight, the most
 that tc_autotune's own candidates go to, leave two pairs to some CTAs and take about twice as long, so the tuner
-has to keep the 12.
+has to keep the 12.  Where the device has no room for the workspace of that many parts (TC_FAULT=nochunks: as if
+so), contexts and batches take at most 8 and compute the same operator.
 """
 import numpy as np
 import pytest
@@ -40,3 +41,29 @@ def test_autotune_times_the_default_counts(prec, tol):
         ctx.close()
     assert so == 12 and 1 <= sc <= 12 and again[0] == 12, (so, sc, again)
     assert np.abs(r1 - r0).max() < tol * np.abs(r0).max() and np.abs(l1 - l0).max() < tol * np.abs(l0).max()
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-13), ("fp32", 1e-5)])
+def test_fewer_chunks_where_memory_is_short(prec, tol, monkeypatch):
+    from paper_2302_07420_gb300.operator import BatchContext
+    p, phi, chi, occ = _case()
+    d_phi, d_chi = torch.from_numpy(phi).cuda(), torch.from_numpy(chi).cuda()
+    outs = []
+    for fault in (None, "nochunks"):
+        if fault:
+            monkeypatch.setenv("TC_FAULT", fault)
+        ctx = _ctx(p, precision=prec)
+        batch = BatchContext([p, p], precision=prec)
+        try:
+            outs += [x.cpu().numpy() for x in ctx.apply(d_phi, d_chi, occ)]
+            r, l = batch.apply([d_phi, d_phi], [d_chi, d_chi], [occ, occ])
+            for k in range(2):
+                outs += [r[k].cpu().numpy(), l[k].cpu().numpy()]
+            if fault:
+                so, sc = ctx.autotune(d_phi, d_chi, occ)
+                assert so <= 8 and sc <= 8, (so, sc)
+        finally:
+            batch.close()
+            ctx.close()
+    for k, x in enumerate(outs):
+        assert np.abs(x - outs[k % 2]).max() < tol * np.abs(outs[k % 2]).max()
