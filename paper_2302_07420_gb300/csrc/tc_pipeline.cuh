@@ -245,7 +245,8 @@ template <typename T, int N> int prepare_kernels(tc_ctx* ctx) {
 // (at most 8 per orbital in k_orbitals).  The uses never overlap in time.
 template <typename T, int N> size_t scratch_needed(const Setup& S, int so_max, int sc_max) {
   const size_t vb = (size_t)vol_bytes<T, N>();
-  // (band contexts: the band points' occupied-pair launch, at most 8 chunks)
+  // (a is at least 12 volumes: k_spec_fwd's two-sided launch takes 8, the merged one of k_hartree_inv 14, for which
+  // run_pipeline looks at the size; band contexts: the band points' occupied-pair launch, at most 8 chunks)
   const size_t a = (size_t)2 * std::max(S.Nk * so_max, S.nkb * 8) * S.no * 6 * vb;
   const size_t b = (size_t)2 * std::max(S.Nk, S.nkb) * S.nb * sc_max * 3 * vb;
   const size_t c = Fit<T, N>::one ? 0 : (size_t)8 * S.Nkt * S.nb * vb;
