@@ -283,9 +283,10 @@ tc_status tc_stage_times(const tc_ctx* ctx, double* ms, int* launches, int n);
 /* tc_pair_kernels -- which kernels the pair stages of this context's applies run (the fused pair
  * chains of Algs. 2, 5, 6, 9, 11, 12; the 3b4 pass of Alg. 10; the occupied-pair stage of Algs. 4,
  * 6, 8, 11).  For each of the three, in that order, info[3 i .. 3 i + 2] =
- *   kind:    0 full transforms, one CTA per item; 1 transforms pruned to the pair-density
- *            support, one CTA per item; 2 transforms on the support (or full) split over a
- *            thread-block cluster, the volumes in the CTAs' distributed shared memory
+ *   kind:    0 full transforms, one CTA per item (up to 16^3 by the kernels of kind 1 with every
+ *            index on the support, TC_FP64 in fixed point as there); 1 transforms pruned to the
+ *            pair-density support, one CTA per item; 2 transforms on the support (or full) split
+ *            over a thread-block cluster, the volumes in the CTAs' distributed shared memory
  *   support: transform points per axis on the spectral side (the box size n for full transforms)
  *   ctas:    CTAs per item (the cluster width; 1 for kinds 0 and 1)
  * The choice follows from the box size, the precision, the Miller span of the spheres (support

@@ -1215,7 +1215,8 @@ tc_status tc_stage_times(const tc_ctx* c, double* ms, int* launches, int n) {
 tc_status tc_pair_kernels(const tc_ctx* c, int* info) {
   if (!c || c->batch) return TC_ERR_STATE;
   if (!info) return TC_ERR_ARG;
-  // the dispatch rule of run_pipeline
+  // the dispatch rule of run_pipeline; kind 0 covers its two forms of the full transforms (up to 16^3 the pruned
+  // kernels' code with every box index on the support, else the full-transform kernels)
   const bool pruned = c->plan_prune_L > 0 && c->pair_support <= c->plan_prune_L;
   const bool dist = !pruned && c->plan_cl_L > 0 && c->pair_support <= c->plan_cl_L;
   for (int k = 0; k < 3; ++k) {

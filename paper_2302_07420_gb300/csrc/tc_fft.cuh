@@ -180,7 +180,7 @@ __host__ __device__ constexpr unsigned long long kfix(int k) {
 // of x.  Else by digits: the product of the low ones, below a quarter of a unit and of either sign, is left out.
 template <int K> __device__ __forceinline__ long long fxmul(long long x) {
   if constexpr (K == KH) {
-    return (x + ((x >> 32) & 1)) >> 1;
+    return (x >> 1) + ((int)(unsigned)x & (int)(x >> 32) & 1);
   } else {
     constexpr Digits k = fx_digits((long long)kfix(K));
     const Digits d = fx_digits(x);

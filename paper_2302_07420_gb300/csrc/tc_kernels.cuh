@@ -93,8 +93,8 @@ template <typename T> struct Params {
   int h3_only;           // occupied-pair stage: the two h3 kinds only (parallel spins, no h6)
   int no_ap;             // pair stages without the work that reads only the antiparallel kernel table
   int u_exp[2];          // values of tabU below 2^u_exp in modulus, per channel (fixed-point transforms' bounds)
-  int fold;              // the pruned pair chains run: Z carries f_q, Y and tn are over tw3b5 (if not 0)
-  int band;              // outputs at band points: no SCF-mesh 3b6 corrections in k_finalize
+  int fold;              // pruned or cluster pair chains run: Z carries f_q, Y and tn are over tw3b5 (if not 0)
+  int band;              // outputs at band points: no SCF-mesh 3b6 corrections in k_local
   int nkb;               // band points (band contexts)
   const double* bandc;   // [nkb][4]: W (3), Gamma_b
   double2* bs;           // [2][nkb][no][nb][13] band correction scalars (tc_band.cuh)
