@@ -38,7 +38,7 @@ SUPPORT = 17
 # right then left: the mean of the two), from one 1-pass capture of the timed apply (the 3 warm-ups and
 # the autotuner's 18 applies skipped); profiles/dram_pruned_kernels_f32_si_k444.md.  Reported only for a
 # captured configuration; cleared whenever the kernel changes.
-CHAIN_TRAFFIC = {(5, False): 10.788e9 + 27.166e9}
+CHAIN_TRAFFIC = {(5, False): 9.473e9 + 26.757e9}
 WORKLOAD_DESC = ("si_k444: FCC a=10.26 bohr, 4x4x4 Gamma-centred k mesh, ecut 7.5 Ha, 24^3 box, "
                  "4 occupied bands, right+left operator")
 

@@ -3,7 +3,7 @@
 // The FP64 pipe of GB300 gives 1.6 additions or fused multiply-adds per clock and SM, the integer
 // pipe 57 64-bit additions and 5.8 64-bit high products (measured, 1024 threads): a 24-point codelet
 // (252 operations, 28 of them products by constants) takes 157 clocks per thread and SM in FP64
-// and about 11 in integers.  So the work volumes of the FP64 pruned kernels hold integers
+// and about 12 in integers.  So the work volumes of the FP64 pruned kernels hold integers
 // v 2^(62 - e), with one exponent e per transform and pass; the products in real space, the spectral
 // multiplications and every accumulator stay in FP64, and FP32 kernels use none of this.
 //
@@ -18,7 +18,8 @@
 // 120 at the worst point, before its conversion to FP64 (boxes of 9^3 to 24^3, both directions, spectra flat
 // and falling off; on the CPU against long double).  With e_3 from bounds as tight as below, that is 0.1e-16
 // to 2.4e-16 of the results' root mean square and 0.7e-16 to 9e-16 at the worst point; the same codelets in
-// FP64 are off by 1.6e-16 to 3.2e-16 and 6e-16 to 42e-16.  (Values that are the same in every pencil are
+// FP64 are off by 1.6e-16 to 3.2e-16 and 6e-16 to 42e-16.  (3x3x3 apply, 24^3: 222 ms with them in integers, 499 in
+// FP64 arithmetic; 2x2x2 gradient 147 and 324.)  (Values that are the same in every pencil are
 // rounded the same way in every pencil: such a coefficient, where only the two ends of the spheres meet, may
 // be off by N^2 / 2 units.)  Bounds come from the 2- and max norms of the real-space factors (k_norms;
 // |sum a b| <= |a|_2 |b|_2) and, for spectra, from sums of upper-rounded floats over the spectrum; factors

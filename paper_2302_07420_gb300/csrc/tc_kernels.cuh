@@ -45,6 +45,7 @@ template <typename T> struct SideArgs {
   cplx<T>* Z;            // [Nk][no][3][N]  -(s2b tw2bx1 grad ket_q + tw3a4 h3a4(q))
   cplx<T>* Y;            // [Nk][nb][3][N]  tw3b3 h1 ket_j - s2b tw2bx2 grad ket_j
   double* cs;            // [nj_out][no][6]: O_qj, X_pp, X_ap (re, im each): 3b6 correction scalars
+                         // (k_corr_scalars overwrites each entry with alpha and omega for k_local)
   cplx<T>* v2;           // [nkb][4]  band points: V2_pp, V2_ap, V3_pp, V3_ap (see tc_band.cuh)
   cplx<T>* bh3a;         // [so][nkb no][3][N]  band points: h3 (3a4 kind) of their occupied orbitals
   cplx<T>* bh3b;         // [so][nkb no][3][N]  band points: h3 (3b kind)

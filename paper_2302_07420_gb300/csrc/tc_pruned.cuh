@@ -235,9 +235,10 @@ template <typename T> inline bool all_terms(const Params<T>& P) {
 // (Algs. 2, 5, 6, 9, 11, 12 and the 2bx terms of Sec. 2.6.3.)  Z comes with f, Y and n over tw3b5, which
 // C takes back: 22 operations per grid point and component instead of 28.
 //
-// What bounds it.  FP64: the products of the parallel-spin pass on the FP64 pipe (half of the time; the
-// transforms run in integers, tc_fixed.cuh): 3x3x3 apply, 24^3, 270.6 -> 129.1 ms.  FP32: the loads of
-// that pass, seven per grid point at the 10 TB/s that L2 gives all SMs together: 4x4x4 76 ms.
+// What bounds it.  FP64: no single pipe; the products of the parallel-spin pass keep the FP64 pipe busy half
+// of the time (the transforms run in integers, tc_fixed.cuh), and the warps wait for instructions (unrolled
+// pencils of 64-bit code), for that pipe's results and at barriers: 3x3x3 apply, 24^3, 270.6 -> 129 ms.  FP32: the
+// latency of that pass's loads, seven per grid point (one point ahead, 18 warps): 4x4x4 88.4 -> 71 ms.
 //
 // Mirrored two-sided launches (P.mirror; Eq. BITCSCFconj).  The left pair density of (output q,
 // partner j) is conj(phi_j^* chi_q) -- the complex conjugate of the right pair density of (output j,
