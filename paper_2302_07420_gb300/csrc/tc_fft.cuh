@@ -122,11 +122,13 @@ template <typename T, int N, int S> __device__ __forceinline__ cplx<T> twiddle(i
     const Digits x = fx_digits(v.x), y = fx_digits(v.y), wr = {(int)(pr >> 32), (int)pr};
     const Digits wi = {S > 0 ? -(int)(pi >> 32) : (int)(pi >> 32), S > 0 ? -(int)pi : (int)pi};
     // |v| <= 2^62 and |w| = 1: the sums of middle products stay below 2^63
-    auto w2 = [](int a, int b, int c, int d) { return (long long)a * b + (long long)c * d; };
+    auto mul = [](int a, int b) { return (long long)a * b; };
     constexpr long long half = 1ll << 29;
-    const long long mr = half + w2(x.l, wr.h, x.h, wr.l) - w2(y.l, wi.h, y.h, wi.l) + (w2(x.l, wr.l, -y.l, wi.l) >> 32);
-    const long long mi = half + w2(x.l, wi.h, x.h, wi.l) + w2(y.l, wr.h, y.h, wr.l) + (w2(x.l, wi.l, y.l, wr.l) >> 32);
-    return {4 * w2(x.h, wr.h, -y.h, wi.h) + (mr >> 30), 4 * w2(x.h, wi.h, y.h, wr.h) + (mi >> 30)};
+    const long long mr = half + (mul(x.l, wr.h) + mul(x.h, wr.l)) - (mul(y.l, wi.h) + mul(y.h, wi.l)) +
+                         ((mul(x.l, wr.l) - mul(y.l, wi.l)) >> 32);
+    const long long mi = half + (mul(x.l, wi.h) + mul(x.h, wi.l)) + (mul(y.l, wr.h) + mul(y.h, wr.l)) +
+                         ((mul(x.l, wi.l) + mul(y.l, wr.l)) >> 32);
+    return {4 * (mul(x.h, wr.h) - mul(y.h, wi.h)) + (mr >> 30), 4 * (mul(x.h, wi.h) + mul(y.h, wr.h)) + (mi >> 30)};
   } else {
     cplx<T> w = tw_load<T>(tw_offset(N) + e);   // exp(-2 pi i e/N)
     if (S > 0) w.y = -w.y;
